@@ -21,6 +21,8 @@
 //      (exact in FP32), which the stage kernel evaluates per velocity.
 // Points with rho <= 0, theta <= 0 or NaN moments set the domain bit of the status word; a Newton
 // correction that stays large sets the Newton bit. No thread waits on another.
+#include <type_traits>
+
 #include "bgk_common.cuh"
 
 namespace bgk {
@@ -370,34 +372,82 @@ __device__ __forceinline__ void assemble_dd(const dfl (&S)[3][3], dfl e0, dfl (&
     M[4] = df_mul(e0, df_scale(m4, 0.5f));
 }
 
+// The solve of one point by L = 1 or 4 lanes. With L = 4 the lanes d = 0, 1, 2 of a point's group form the
+// 1-D sums of axis d (the bulk of the work, and independent by axis) and the partial sums of the moment
+// components are shared out too; everything else is computed by all four alike, so that they stay in
+// step, and lane 0 writes. Every sum is formed in the same order either way.
+template <int L>
 __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
 {
+    const int sub = L == 1 ? 0 : (threadIdx.x & 3);
+    const unsigned grp = L == 1 ? 0u : 0xFu << (threadIdx.x & 28);  // this point's lanes
+    const bool writer = sub == 0;
+    // v of lane d of the group
+    auto from = [&](float v, int d) { return __shfl_sync(grp, v, d, 4); };
 
     // 1. moments: exact sum of the FP32 partials (or the FP64 moments of the all-FP64 form)
     double Q[5];
+    if (A.Qin) {
 #pragma unroll
-    for (int c = 0; c < 5; c++) {
-        if (A.Qin) {
+        for (int c = 0; c < 5; c++)
             Q[c] = A.Qin[(int64_t)pt * 5 + c];
-            continue;
+    } else {
+        // kU groups' loads in flight at a time (a batch's 32^3-velocity member has 128 groups: 640 loads, whose
+        // latencies were the batched solve's longest part, 0.33 -> 0.13 ms per launch of the Sod ensemble).
+        // With four lanes component c is lane c mod 4's (lane 0: 0 and 4).
+        constexpr int kU = 4, kC = L == 1 ? 5 : 2;
+        const float *p[kC];
+        float hi[kC], lo[kC];
+#pragma unroll
+        for (int c = 0; c < kC; c++) {
+            const int comp = L == 1 ? c : (c == 0 ? sub : (sub == 0 ? 4 : sub));
+            p[c] = A.partial + (int64_t)comp * A.npts + pt;
+            hi[c] = lo[c] = 0.f;
         }
-        float hi = 0.f, lo = 0.f;
-        const float *p = A.partial + (int64_t)c * A.npts + pt;
-        for (int g = 0; g < A.ngroups; g++) {
-            float s, e;
-            two_sum(hi, __ldg(p + (int64_t)g * 5 * A.npts), s, e);
-            hi = s;
-            lo += e;
+        const int64_t gs = (int64_t)5 * A.npts;
+        int g = 0;
+        auto take = [&](auto n_c) {
+            constexpr int N = decltype(n_c)::value;
+            float v[N][kC];
+#pragma unroll
+            for (int k = 0; k < N; k++)
+#pragma unroll
+                for (int c = 0; c < kC; c++)
+                    v[k][c] = __ldg(p[c] + (g + k) * gs);
+#pragma unroll
+            for (int k = 0; k < N; k++)
+#pragma unroll
+                for (int c = 0; c < kC; c++) {
+                    float s, e;
+                    two_sum(hi[c], v[k][c], s, e);
+                    hi[c] = s;
+                    lo[c] += e;
+                }
+            g += N;
+        };
+        while (g + kU <= A.ngroups)
+            take(std::integral_constant<int, kU>{});
+        while (g < A.ngroups)
+            take(std::integral_constant<int, 1>{});
+        if (L > 1) {
+            const float h0 = hi[0], l0 = lo[0], h4 = hi[1], l4 = lo[1];
+#pragma unroll
+            for (int c = 0; c < 5; c++)
+                Q[c] = (double)from(c < 4 ? h0 : h4, c & 3) + (double)from(c < 4 ? l0 : l4, c & 3);
+        } else {
+#pragma unroll
+            for (int c = 0; c < 5; c++)
+                Q[c] = (double)hi[c % kC] + (double)lo[c % kC];
         }
-        Q[c] = (double)hi + (double)lo;
     }
     if (!A.Qin) {  // the FP32 kernels sum in the grid-index basis
         const double mu[5] = {Q[0], Q[1], Q[2], Q[3], Q[4]};
         index_to_moments(mu, A.v0, A.dv, A.n, Q);
     }
+    if (writer)
 #pragma unroll
-    for (int c = 0; c < 5; c++)
-        A.Q[(int64_t)pt * 5 + c] = Q[c];
+        for (int c = 0; c < 5; c++)
+            A.Q[(int64_t)pt * 5 + c] = Q[c];
 
     const double rho = Q[0], irho = 1.0 / rho;
     const double u[3] = {Q[1] * irho, Q[2] * irho, Q[3] * irho};
@@ -405,6 +455,8 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
     const double thc = (Q[4] * irho - 0.5 * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2])) * (A.vdim == 2 ? 1.0 : 2.0 / 3.0);
     float *par = A.param + (int64_t)pt * kParamStride;
     if (!(rho > 0.0) || !(thc > 0.0) || !isfinite(rho) || !isfinite(thc)) {
+        if (!writer)
+            return;
         atomicOr(A.err, kErrDomain);
         par[0] = -1e30f;  // g = 0 at this point
         for (int c = 1; c < kParamStride; c++)
@@ -462,6 +514,8 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
         // in FP32: the steps accumulate in da and are added to the FP64 alpha once at the end
         float J[5][5];
         bool haveJ = false;
+        auto pick = [&](auto x, auto y, auto z) { return sub == 0 ? x : (sub == 1 ? y : z); };  // this lane's axis
+        const int nax = pick(A.n[0], A.n[1], A.n[2]);
         const int it32min = warm ? A.it32 : max(A.it32, 4);
         // the targets, grid and starting alpha as double-float pairs (the refinement's operands); their
         // high parts are the FP32 loop's (alpha_1..3 = 0 and alpha_4 = -1 are exact)
@@ -485,9 +539,20 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
         }
         for (int it = 0; it < 30; it++) {
             float S[3][5];
+            if constexpr (L == 1) {
     #pragma unroll
-            for (int d = 0; d < 3; d++)
-                sums32(a0[1 + d] + da[1 + d], -(a0[4] + da[4]), c0f[d], hf[d], A.n[d], dvf[d], S[d]);
+                for (int d = 0; d < 3; d++)
+                    sums32(a0[1 + d] + da[1 + d], -(a0[4] + da[4]), c0f[d], hf[d], A.n[d], dvf[d], S[d]);
+            } else {  // lane 3 repeats axis 2
+                float So[5];
+                sums32(pick(a0[1] + da[1], a0[2] + da[2], a0[3] + da[3]), -(a0[4] + da[4]),
+                       pick(c0f[0], c0f[1], c0f[2]), pick(hf[0], hf[1], hf[2]), nax, pick(dvf[0], dvf[1], dvf[2]), So);
+    #pragma unroll
+                for (int d = 0; d < 3; d++)
+    #pragma unroll
+                    for (int m = 0; m < 5; m++)
+                        S[d][m] = from(So[m], d);
+            }
             float M[5];
             assemble<float>(S, expf(a0[0] + da[0]), M, J);
             haveJ = true;
@@ -524,7 +589,8 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
         for (int m = 0; m < 5; m++)
             ald[m] = df_add(ald[m], {da[m], 0.f});
         if (!haveJ) {
-            atomicOr(A.err, kErrNewton);
+            if (writer)
+                atomicOr(A.err, kErrNewton);
             return;
         }
 
@@ -535,16 +601,31 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
         // FP64 rate is 1/60 of its FP32 rate, and the same residual in FP64 took 58 % of this kernel.
         const int it64min = warm ? A.it64 : max(A.it64, 2);
         for (int it = 0; it < 4; it++) {
-            dfl S[3][3], E2[3], lnp = {0.f, 0.f};
+            dfl S[3][3], lnp = {0.f, 0.f};
             const dfl beta = df_neg(ald[4]);
+            if constexpr (L == 1) {
+                dfl E2[3];
     #pragma unroll
-            for (int d = 0; d < 3; d++)
-                E2[d] = d > 0 && hd[d].hi == hd[d - 1].hi && hd[d].lo == hd[d - 1].lo
-                            ? E2[d - 1]
-                            : df_exp(df_mul(ald[4], df_mul(hd[d], hd[d])));
+                for (int d = 0; d < 3; d++)
+                    E2[d] = d > 0 && hd[d].hi == hd[d - 1].hi && hd[d].lo == hd[d - 1].lo
+                                ? E2[d - 1]
+                                : df_exp(df_mul(ald[4], df_mul(hd[d], hd[d])));
     #pragma unroll
-            for (int d = 0; d < 3; d++)
-                lnp = df_add(lnp, sums_dd(ald[1 + d], beta, c0d[d], hd[d], A.n[d], dvd[d], E2[d], S[d]));
+                for (int d = 0; d < 3; d++)
+                    lnp = df_add(lnp, sums_dd(ald[1 + d], beta, c0d[d], hd[d], A.n[d], dvd[d], E2[d], S[d]));
+            } else {  // lane 3 repeats axis 2
+                dfl So[3];
+                const dfl ho = pick(hd[0], hd[1], hd[2]);
+                const dfl lo = sums_dd(pick(ald[1], ald[2], ald[3]), beta, pick(c0d[0], c0d[1], c0d[2]), ho, nax,
+                                       pick(dvd[0], dvd[1], dvd[2]), df_exp(df_mul(ald[4], df_mul(ho, ho))), So);
+    #pragma unroll
+                for (int d = 0; d < 3; d++) {
+    #pragma unroll
+                    for (int m = 0; m < 3; m++)
+                        S[d][m] = {from(So[m].hi, d), from(So[m].lo, d)};
+                    lnp = df_add(lnp, {from(lo.hi, d), from(lo.lo, d)});
+                }
+            }
             dfl M[5];
             assemble_dd(S, df_exp(df_add(ald[0], lnp)), M);  // the peaks' factors with alpha_0
             if (A.vdim == 2)
@@ -561,7 +642,8 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
                     Jw[m][q] = J[m][q];
             }
             if (!solve5<float>(Jw, r, dx)) {
-                atomicOr(A.err, kErrNewton);
+                if (writer)
+                    atomicOr(A.err, kErrNewton);
                 return;
             }
             float cf = 0.f;
@@ -582,9 +664,12 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
     }
     const double beta = -al[4];
     if (!(beta > 0.0) || !isfinite(al[0] + al[1] + al[2] + al[3]) || corr >= 1e-6) {
-        atomicOr(A.err, kErrNewton);
+        if (writer)
+            atomicOr(A.err, kErrNewton);
         return;
     }
+    if (!writer)
+        return;
 
     // 3. outputs: perturbed state and the stage kernel's exponent in the raw velocity
     const double a[3] = {al[1], al[2], al[3]};
@@ -682,31 +767,34 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
     }
 }
 
-// Resident CTAs of 128 threads per SM the register allocation is sized for. The solve is bound by the
-// latency of its FP32 and FP64 chains and by the FP64 pipe, which more resident warps keep busier:
-// 8 CTAs (64 registers, spilling to L1) run the 262,144-point solves of the planar and Taylor-Green
-// workloads 10-17 % faster than 4 (128 registers); the batched solve, whose arguments come from
-// global memory, runs best at 4.
-#ifndef BGK_NEWTON_MINCTAS
-#define BGK_NEWTON_MINCTAS 8
-#endif
-#ifndef BGK_NEWTON_BATCH_MINCTAS
-#define BGK_NEWTON_BATCH_MINCTAS 4
-#endif
+// The two forms of the solve, by the number of points (128-thread CTAs on 152 SMs; us per launch alone,
+// before -> now, with the partial sums' loads four groups at a time):
+//   up to 19,456   one wave of latency: four lanes share a point, 4 CTAs per SM leave the 128 registers that
+//                  avoid spills (72 points 44 -> 23; 6,000 points 80 -> 39; 12,000 points 90 -> 47);
+//   beyond         the FP64 pipe (a warp instruction per 16 clocks and SM; some 230 per point in the set-up
+//                  and the outputs) and the chains' latency: a thread per point, 8 CTAs (64 registers,
+//                  spilling to L1) keep it busiest (262,144 points 170 -> 164; 4 CTAs 198, four lanes per
+//                  point 512). Between 19,456 and 77,824 points 4 CTAs are faster alone (20,160 points 99
+//                  against 107) but slower where other work shares the SMs, since they hold twice the
+//                  registers: three contexts of 20,160 points stepped in turn 5.59 against 5.42 ms per pass.
+// The batched solve, whose arguments come from global memory, runs best at 4 CTAs.
+constexpr int kNewtonThreads = 128, kLanePoints = 152 * 4 * kNewtonThreads / 4;
 
-__global__ void __launch_bounds__(128, BGK_NEWTON_MINCTAS) k_newton(const NewtonArgs A)
+template <int L, int MINCTAS>
+__global__ void __launch_bounds__(kNewtonThreads, MINCTAS) k_newton(const NewtonArgs A)
 {
-    const int pt = blockIdx.x * blockDim.x + threadIdx.x;
+    const int pt = (blockIdx.x * blockDim.x + threadIdx.x) / L;
     if (pt < A.npts)
-        newton_point(A, pt);
+        newton_point<L>(A, pt);
 }
 
-// Batched solve over the points of many independent problems: thread per point, the problem found
+// Batched solve over the points of many independent problems: L lanes per point, the problem found
 // by a binary search over the point prefix sums pt_start[0..n].
-__global__ void __launch_bounds__(128, BGK_NEWTON_BATCH_MINCTAS) k_newton_batch(const NewtonArgs *__restrict__ args,
-                                                      const int *__restrict__ pt_start, int n)
+template <int L>
+__global__ void __launch_bounds__(kNewtonThreads, 4) k_newton_batch(const NewtonArgs *__restrict__ args,
+                                                                    const int *__restrict__ pt_start, int n)
 {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    const int g = (blockIdx.x * blockDim.x + threadIdx.x) / L;
     if (g >= pt_start[n])
         return;
     int lo = 0, hi = n;
@@ -717,21 +805,27 @@ __global__ void __launch_bounds__(128, BGK_NEWTON_BATCH_MINCTAS) k_newton_batch(
         else
             hi = mid;
     }
-    newton_point(args[lo], g - pt_start[lo]);
+    newton_point<L>(args[lo], g - pt_start[lo]);
 }
+
+static int newton_ctas(int points, int lanes) { return (int)(((int64_t)points * lanes + kNewtonThreads - 1) / kNewtonThreads); }
 
 cudaError_t launch_newton_batch(const NewtonArgs *d_args, const int *d_pt_start, int n, int total_pts,
                                 cudaStream_t s)
 {
-    const int threads = 128;
-    k_newton_batch<<<(total_pts + threads - 1) / threads, threads, 0, s>>>(d_args, d_pt_start, n);
+    if (total_pts <= kLanePoints)
+        k_newton_batch<4><<<newton_ctas(total_pts, 4), kNewtonThreads, 0, s>>>(d_args, d_pt_start, n);
+    else
+        k_newton_batch<1><<<newton_ctas(total_pts, 1), kNewtonThreads, 0, s>>>(d_args, d_pt_start, n);
     return cudaGetLastError();
 }
 
 cudaError_t launch_newton(const NewtonArgs &A, cudaStream_t s)
 {
-    const int threads = 128;
-    k_newton<<<(A.npts + threads - 1) / threads, threads, 0, s>>>(A);
+    if (A.npts <= kLanePoints)
+        k_newton<4, 4><<<newton_ctas(A.npts, 4), kNewtonThreads, 0, s>>>(A);
+    else
+        k_newton<1, 8><<<newton_ctas(A.npts, 1), kNewtonThreads, 0, s>>>(A);
     return cudaGetLastError();
 }
 
