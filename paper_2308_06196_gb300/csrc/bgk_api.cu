@@ -40,8 +40,9 @@ cudaError_t launch_limit64(double *f, int nvt, int E, int NP, int N1, int dim, c
                            cudaStream_t s);
 cudaError_t launch_wall(const WallArgs &A, bool fp64, const void *w, const void *xi, cudaStream_t s);
 cudaError_t launch_moments64(const Moments64Args &A, cudaStream_t s);
-cudaError_t launch_init64(double *f, const double *prim, const double *xi, const float *gmask, int nvt, int E, int NP,
-                          int nslots, int vdim, int *err, cudaStream_t s);
+cudaError_t launch_init64(double *f, const double *prim, double *par, double *tab, const Table64Args &T,
+                          const float *gmask, int nvt, int npts, int vdim, int *err, cudaStream_t s);
+cudaError_t launch_table64(double *tab, const double *par, const Table64Args &T, int npts, cudaStream_t s);
 cudaError_t launch_convert64(bool to_device, double *f, double *st, const int *slotk, int nvt, int E, int NP,
                              int64_t nvel, int p0, int npt, cudaStream_t s);
 cudaError_t launch_f_distance(const void *a, bool a64, const void *b, bool b64, const int *slotk, int nvt, int E,
@@ -136,6 +137,10 @@ void build_ops(int p, Ops &op, Ops64 &o64, double *xg_out)
         o64.gl[i] = gl[i];
         o64.gr[i] = gr[i];
         o64.wq[i] = 0.5 * W[i];
+        for (int j = 0; j < n; j++) {
+            o64.DL[i][j] = D[i][j] - gl[i] * lm[j];
+            o64.DR[i][j] = D[i][j] - gr[i] * lp[j];
+        }
     }
     for (int i = 0; i < n; i++) {
         for (int j = 0; j < n; j++) {
@@ -195,6 +200,7 @@ struct bgk_ctx {
     // all-FP64 form
     int prec = BGK_FP32_SPLIT;
     double *fA64 = nullptr, *pool64 = nullptr, *xi64 = nullptr, *wpsi64 = nullptr, *ghost64 = nullptr, *par64 = nullptr;
+    double *etab64 = nullptr;  // [n_x][sum_d n_d] 1-D factors of the Maxwellian (all-FP64 form)
     // diffuse walls and body force
     bool has_wall = false, has_force = false;
     // exchange faces (x faces shared with a neighbouring subdomain): the halos, [nvt][E_face][NP][32]
@@ -415,6 +421,19 @@ Moments64Args moments64_args(bgk_ctx *c)
     return M;
 }
 
+Table64Args table64_args(const bgk_ctx *c)
+{
+    Table64Args T{};
+    for (int d = 0; d < 3; d++) {
+        T.v0[d] = c->vlo[d];
+        T.dv[d] = c->dv[d];
+        T.n[d] = c->nv[d];
+    }
+    T.mi = c->mi;
+    T.nslots = c->nslots;
+    return T;
+}
+
 // Moments of the state f^n and its conservative Maxwellian (after bgk_set_state / bgk_set_f). have_q:
 // Q was formed with the state (the initial sampling's separable moments) and the Newton solve starts
 // from the sampled Maxwellian itself; otherwise a moments pass over f and a cold solve.
@@ -518,6 +537,7 @@ int enqueue_step64(bgk_ctx *c, double dt, cudaStream_t s, const std::vector<int>
             if (rc)
                 return rc;
         }
+        CK(launch_table64(c->etab64, c->par64, table64_args(c), (int)c->npts, s));
         for (int q = 0; q < C; q++) {
             const Chunk &ch = c->chunks[q];
             double *Aq = chunk_ptr64(c, c->fA64, ch.vt0);
@@ -529,7 +549,9 @@ int enqueue_step64(bgk_ctx *c, double dt, cudaStream_t s, const std::vector<int>
             A.dst = st == 0 ? s1 : (st == 1 ? s2 : Aq);
             A.xi = c->xi64;
             A.ghost = c->ghost64;
-            A.par = c->par64;
+            A.etab = c->etab64;
+            A.tab = table64_args(c);
+            A.toct = c->toct;
             A.rhow = c->rhow64;
             A.fpar = c->fpar64;
             A.nfmax = c->nfmax;
@@ -705,7 +727,7 @@ void bgk_destroy(bgk_ctx *c)
         cudaEventDestroy(ev.b);
     }
     void *bufs[] = {c->fA, c->pool, c->xi, c->mi, c->vtab, c->toct, c->wpsi, c->gmask, c->ghost, c->slotk_d, c->partial,
-                    c->param, c->Q, c->prim, c->prim_in, c->err, c->fA64, c->pool64, c->xi64,
+                    c->param, c->Q, c->prim, c->prim_in, c->err, c->fA64, c->pool64, c->xi64, c->etab64,
                     c->wpsi64, c->ghost64, c->par64, c->rhow32, c->fpar32, c->w32, c->rhow64,
                     c->fpar64, c->w64, c->itau64, c->met, c->fnm, c->iwj, c->ftab, c->fbase, c->wn64,
                     c->ja64, c->ijac64, c->fnm64, c->wlist, c->wnu, c->rhowu32, c->rhowu64,
@@ -921,6 +943,7 @@ int bgk_create(const bgk_mesh *mesh, int p, const bgk_vgrid *vg, double tau, con
     const int64_t need = (fA + (int64_t)(c->chunks.size() + 1) * c->chunk_floats) * c->esize +
                          (int64_t)c->max_groups * 5 * c->npts * 4 + c->npts * (5 * 8 * 3 + kParamStride * 4) +
                          (int64_t)c->nslots * 4 * 25 +
+                         (c->prec == BGK_FP64 ? c->npts * 8 * (c->nv[0] + c->nv[1] + c->nv[2]) : 0) +
                          (c->has_exchange ? 2 * (int64_t)c->nvt * c->ne[1] * c->ne[2] * c->NP * kWarp * 4 : 0);
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess)
@@ -942,6 +965,7 @@ int bgk_create(const bgk_mesh *mesh, int p, const bgk_vgrid *vg, double tau, con
         AL(c->wpsi64, 5 * c->nslots);
         AL(c->ghost64, 6 * c->nslots);
         AL(c->par64, c->npts * 5);
+        AL(c->etab64, c->npts * (c->nv[0] + c->nv[1] + c->nv[2]));
         if (c->opts.mu_ref > 0.0)
             AL(c->itau64, c->npts);
     } else {
@@ -1124,8 +1148,8 @@ static int set_state_impl(bgk_ctx *c, const double *prim, cudaMemcpyKind kind)
 {
     CK(cudaMemcpyAsync(c->prim_in, prim, c->npts * 5 * sizeof(double), kind, c->stream));
     if (c->prec == BGK_FP64)
-        CK(launch_init64(c->fA64, c->prim_in, c->xi64, c->gmask, c->nvt, c->E, c->NP, c->nslots, c->vdim, c->err,
-                         c->stream));
+        CK(launch_init64(c->fA64, c->prim_in, c->par64, c->etab64, table64_args(c), c->gmask, c->nvt, (int)c->npts,
+                         c->vdim, c->err, c->stream));
     else
         CK(launch_init_maxwellian(c->fA, c->prim_in, c->mi, c->gmask, c->nslots, c->nvt, c->E, c->NP, c->nv, c->vlo,
                                   c->dv, c->err, c->Q, c->prim, c->stream));

@@ -150,18 +150,28 @@ inline void newton_axis(NewtonArgs &N, int d, double v0, double dv, int n)
 // FR reference operators in FP64 for the plain all-FP64 form (Sec. 2.1, Eqs. 7-9).
 struct Ops64 {
     double D[kMaxN1][kMaxN1];
+    double DL[kMaxN1][kMaxN1], DR[kMaxN1][kMaxN1];  // D - gl (x) lm, D - gr (x) lp (one inflow side each)
     double lm[kMaxN1], lp[kMaxN1];
     double gl[kMaxN1], gr[kMaxN1];
     double wq[kMaxN1];  // Gauss-Legendre weights / 2
 };
 
-// One launch of the plain FP64 stage kernel over one velocity chunk (thread per degree of freedom).
+// The velocity grid of the plain FP64 form's 1-D Maxwellian factors.
+struct Table64Args {
+    double v0[3], dv[3];
+    int n[3];
+    const float *mi;  // [3][nslots] centred grid index of every slot (StageArgs::mi)
+    int nslots;
+};
+
+// One launch of the plain FP64 stage kernel over one velocity chunk.
 struct Stage64Args {
     const double *src, *fn;
     double *dst;
     const double *xi;      // [3][nslots]
     const double *ghost;   // [6][nslots]
-    const double *par;     // [n_x][5] (C, U', 1/(2 theta')) of the conservative Maxwellian
+    const double *etab;    // [n_x][n_x-axis + n_y + n_z] the Maxwellian's 1-D factors (k64_table)
+    Table64Args tab;
     const double *rhow;    // [6][nfmax][N1^2] diffuse-wall densities, or null
     const double *fpar;    // [n_x][5] body-force polynomial, or null
     int nfmax;
@@ -171,6 +181,7 @@ struct Stage64Args {
     double h[3];
     int N1, NP;
     int vt0, nvt, nslots;
+    const unsigned char *toct;  // [nvt] sign octant of every tile (bit d: xi_d >= 0)
     double an, b, dt, inv_tau;
     const double *itau;    // [n_x] per-point 1/tau (variable collision time), or null: inv_tau
     // curvilinear hexahedra (null on the affine mesh): the metric rows Ja^d of every node [n_x][3][3]

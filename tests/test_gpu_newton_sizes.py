@@ -1,6 +1,7 @@
-"""The Newton solve's forms by point count (four lanes per point, a thread per point) form every sum in the same order, so they give the same bits: a line whose elements are copies of one
-another is solved at point counts on both sides of the limit and with ragged last warps, and every
-element must agree with the shortest line's, exactly."""
+"""The Newton solve's forms by point count (four lanes per point, a thread per point) form every sum in the
+same order, so they give the same bits: a line whose elements are copies of one another is solved at point
+counts on both sides of the limit and with ragged last warps, and every element must agree with the
+shortest line's, exactly."""
 import numpy as np
 import pytest
 
