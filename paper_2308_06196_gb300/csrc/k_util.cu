@@ -1,19 +1,27 @@
 // k_util.cu -- set-up and data-movement kernels of libbgk: sampling the initial Maxwellian into the
 // device layout, and converting f between the host order [point][velocity] (FP64) and the device
 // tile layout f[vt][e][i][lane] (FP32).
+#include <algorithm>
+
 #include "bgk_common.cuh"
 
 namespace bgk {
 
 // Sample the continuous Maxwellian (Sec. 2, Eq. 4, velocity dimension m = 3, or 2 when nz = 1: the
-// one z node has factor 1 and U_z takes no part) of every point's primitive state into f. One CTA per
-// element: the separable factors exp(-(xi_d - U_d)^2 / (2 theta)) of the element's points are tabulated
-// once in shared memory as FP32 (the exponent in FP64, split into an integer power of two and a
-// remainder in [-1/2, 1/2] whose 2^r is taken in FP32: within a few FP32 ulp at any exponent), then every
-// (tile, node, lane) value is the product C * Ex * Ey * Ez. Writes 0 on padded slots.
+// one z node has factor 1 and U_z takes no part) of every point's primitive state into f. A CTA owns PB
+// consecutive points (of as many elements as that takes) and a run of velocity tiles: the separable
+// factors exp(-(xi_d - U_d)^2 / (2 theta)) of its points are tabulated once in shared memory as FP32 (the
+// exponent in FP64, split into an integer power of two and a remainder in [-1/2, 1/2] whose 2^r is taken
+// in FP32: within a few FP32 ulp at any exponent), then every (tile, point, lane) value is the product
+// (C Ex) Ey Ez. Writes 0 on padded slots.
 // Q (when not null): the discrete moments (Eq. 2 with Eq. 12) of every point's sampled Maxwellian in
 // FP64, from the 1-D trapezoid sums of its tabulated factors (the grid is a tensor product): they differ
 // from the moments of the stored FP32 values only by the rounding of the products.
+// Bound: the tables by the FP64 pipe (a warp instruction per 16 clocks, whatever its active lanes), the
+// values by the writing of f. One CTA per element left most lanes of the table and moment work idle at
+// four points per element, and a small mesh's tiles to a few CTAs. 65,536 line elements at p = 3, 32^2
+// velocities (1.1 GB of f): 3.24 ms before, 1.00 now; 128^2 quadrilaterals 1.37 -> 1.00; 16^3
+// hexahedra, 24^3 velocities (14.5 GB) 3.34 -> 3.25.
 __device__ __forceinline__ float exp_split(double x)
 {
     const double y = x * 1.4426950408889634;  // log2(e)
@@ -21,34 +29,33 @@ __device__ __forceinline__ float exp_split(double x)
     return ldexpf(exp2f((float)(y - n)), (int)n);
 }
 
-// Resident CTAs per SM the register allocation is sized for (4, 5 and 6 measured within 2 % of each other)
-#ifndef BGK_INIT_MINCTAS
-#define BGK_INIT_MINCTAS 5
-#endif
-
-__global__ void __launch_bounds__(256, BGK_INIT_MINCTAS)
+__global__ void __launch_bounds__(256, 4)
     k_init_maxwellian(float *__restrict__ f, const double *__restrict__ prim, const float *__restrict__ mi,
-                      const float *__restrict__ gmask, int nslots, int nvt, int E, int NP, int nx, int ny, int nz,
-                      double v0x, double v0y, double v0z, double dvx, double dvy, double dvz, int *err,
+                      const float *__restrict__ gmask, int nslots, int nvt, int npts, int PB, int tiles, int nx, int ny,
+                      int nz, double v0x, double v0y, double v0z, double dvx, double dvy, double dvz, int *err,
                       double *__restrict__ Q, double *__restrict__ warm)
 {
     const double hm = nz == 1 ? 1.0 : 1.5;  // m / 2
-    extern __shared__ double ith[];          // [NP] -1 / (2 theta) of the element's points, then
-    float *tab = reinterpret_cast<float *>(ith + NP);  // [NP][nx + ny + nz + 1]
-    const int e = blockIdx.x;
-    const int ntab = nx + ny + nz + 1;
+    const int ntab = nx + ny + nz + 1;       // per point: 0 (padded slots), then the factors by axis
+    extern __shared__ double ith[];          // [PB] -1 / (2 theta) of the CTA's points,
+    double *S = ith + PB;                    // [PB][3][3] 1-D sums,
+    float *cn = reinterpret_cast<float *>(S + 9 * PB);  // [PB] normalisations,
+    float *tab = cn + PB;                    // [PB][ntab]
+    const int p0 = blockIdx.x * PB, np = min(PB, npts - p0);
+    const bool first = blockIdx.y == 0;      // writes the points' moments and warm starts
     // per point: the normalisation rho (2 pi theta)^(-m/2) and -1 / (2 theta) (one division per point)
-    for (int i = threadIdx.x; i < NP; i += blockDim.x) {
-        const double *s = prim + ((int64_t)e * NP + i) * 5;
+    for (int i = threadIdx.x; i < np; i += blockDim.x) {
+        const double *s = prim + (int64_t)(p0 + i) * 5;
         const double rho = s[0], th = s[4];
         const bool ok = rho > 0.0 && th > 0.0;
         if (!ok)
             atomicOr(err, kErrDomain);
         ith[i] = ok ? -0.5 / th : 0.0;
         const double C = rho * pow(2.0 * 3.14159265358979323846 * th, -hm);
-        tab[i * ntab] = ok ? (float)C : 0.f;
-        if (warm && ok) {  // the first Newton solve's start: this Maxwellian, (ln C, U, theta)
-            double *wp = warm + ((int64_t)e * NP + i) * 5;
+        cn[i] = ok ? (float)C : 0.f;
+        tab[i * ntab] = 0.f;
+        if (warm && ok && first) {  // the first Newton solve's start: this Maxwellian, (ln C, U, theta)
+            double *wp = warm + (int64_t)(p0 + i) * 5;
             wp[0] = log(C);
             wp[1] = s[1];
             wp[2] = s[2];
@@ -57,9 +64,9 @@ __global__ void __launch_bounds__(256, BGK_INIT_MINCTAS)
         }
     }
     __syncthreads();
-    for (int q = threadIdx.x; q < NP * (ntab - 1); q += blockDim.x) {
+    for (int q = threadIdx.x; q < np * (ntab - 1); q += blockDim.x) {
         const int i = q / (ntab - 1), t = 1 + q % (ntab - 1);
-        const double *s = prim + ((int64_t)e * NP + i) * 5;
+        const double *s = prim + (int64_t)(p0 + i) * 5;
         const double a = ith[i];
         float v;
         if (t <= nx) {
@@ -77,66 +84,76 @@ __global__ void __launch_bounds__(256, BGK_INIT_MINCTAS)
         tab[i * ntab + t] = a == 0.0 ? 0.f : v;
     }
     __syncthreads();
-    if (Q)
-        for (int i = threadIdx.x; i < NP; i += blockDim.x) {
-            const float *t = tab + i * ntab;
-            const int n[3] = {nx, ny, nz};
-            const double v0[3] = {v0x, v0y, v0z}, dv[3] = {dvx, dvy, dvz};
-            double S[3][3];
-            int off = 1;
-            for (int d = 0; d < 3; d++) {
-                S[d][0] = S[d][1] = S[d][2] = 0.0;
-                if (n[d] == 1) {  // the absent u_z: one node at 0 of unit weight
-                    S[d][0] = (double)t[off];
-                } else {
-                    for (int k = 0; k < n[d]; k++) {
-                        const double x = v0[d] + k * dv[d];
-                        const double a = (k == 0 || k == n[d] - 1 ? 0.5 * dv[d] : dv[d]) * (double)t[off + k];
-                        S[d][0] += a;
-                        S[d][1] = fma(x, a, S[d][1]);
-                        S[d][2] = fma(x * x, a, S[d][2]);
-                    }
+    if (Q && first) {
+        // the 1-D sums of every (point, axis) by a thread of its own, then the points' moments
+        for (int q = threadIdx.x; q < 3 * np; q += blockDim.x) {
+            const int d = q / np, i = q % np;
+            const int n = d == 0 ? nx : (d == 1 ? ny : nz);
+            const double v0 = d == 0 ? v0x : (d == 1 ? v0y : v0z), dv = d == 0 ? dvx : (d == 1 ? dvy : dvz);
+            const float *t = tab + i * ntab + 1 + (d > 0 ? nx : 0) + (d > 1 ? ny : 0);
+            double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+            if (n == 1) {  // the absent u_z: one node at 0 of unit weight
+                s0 = (double)t[0];
+            } else {
+                for (int k = 0; k < n; k++) {
+                    const double x = v0 + k * dv;
+                    const double a = (k == 0 || k == n - 1 ? 0.5 * dv : dv) * (double)t[k];
+                    s0 += a;
+                    s1 = fma(x, a, s1);
+                    s2 = fma(x * x, a, s2);
                 }
-                off += n[d];
             }
-            const double C = (double)t[0];
-            double *q = Q + ((int64_t)e * NP + i) * 5;
-            q[0] = C * S[0][0] * S[1][0] * S[2][0];
-            q[1] = C * S[0][1] * S[1][0] * S[2][0];
-            q[2] = C * S[0][0] * S[1][1] * S[2][0];
-            q[3] = C * S[0][0] * S[1][0] * S[2][1];
-            q[4] = 0.5 * C * (S[0][2] * S[1][0] * S[2][0] + S[0][0] * S[1][2] * S[2][0] + S[0][0] * S[1][0] * S[2][2]);
+            double *o = S + (i * 3 + d) * 3;
+            o[0] = s0;
+            o[1] = s1;
+            o[2] = s2;
         }
+        __syncthreads();
+        for (int i = threadIdx.x; i < np; i += blockDim.x) {
+            const double(*s)[3] = reinterpret_cast<const double(*)[3]>(S + 9 * i);
+            const double C = (double)cn[i];
+            double *q = Q + (int64_t)(p0 + i) * 5;
+            q[0] = C * s[0][0] * s[1][0] * s[2][0];
+            q[1] = C * s[0][1] * s[1][0] * s[2][0];
+            q[2] = C * s[0][0] * s[1][1] * s[2][0];
+            q[3] = C * s[0][0] * s[1][0] * s[2][1];
+            q[4] = 0.5 * C * (s[0][2] * s[1][0] * s[2][0] + s[0][0] * s[1][2] * s[2][0] + s[0][0] * s[1][0] * s[2][2]);
+        }
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < np * nx; q += blockDim.x)  // the normalisation into the x factors
+        tab[(q / nx) * ntab + 1 + q % nx] *= cn[q / nx];
+    __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     // the tile's table columns (1 + k_x, 1 + n_x + k_y, 1 + n_x + n_y + k_z) from the centred index table
-    // (k_d = (m_d + n_d - 1) / 2, exact) and its mask; the next tile's are loaded while this one is written
-    auto slot_cols = [&](int vt, int &cx, int &cy, int &cz, float &gm) {
+    // (k_d = (m_d + n_d - 1) / 2, exact), column 0 on padded slots; the next tile's are loaded while this one
+    // is written
+    auto slot_cols = [&](int vt, int &cx, int &cy, int &cz) {
         const int slot = vt * kWarp + lane;
         cx = 1 + __float2int_rn(0.5f * (__ldg(mi + slot) + (float)(nx - 1)));
         cy = 1 + nx + __float2int_rn(0.5f * (__ldg(mi + nslots + slot) + (float)(ny - 1)));
         cz = 1 + nx + ny + __float2int_rn(0.5f * (__ldg(mi + 2 * nslots + slot) + (float)(nz - 1)));
-        gm = __ldg(gmask + slot);
+        if (__ldg(gmask + slot) == 0.f)
+            cx = 0;
     };
+    const int vt0 = blockIdx.y * tiles, vt1 = min(vt0 + tiles, nvt);
+    if (vt0 >= vt1)
+        return;
     int cx, cy, cz;
-    float gm;
-    slot_cols(0, cx, cy, cz, gm);
-    for (int vt = 0; vt < nvt; vt++) {
-        int nx_, ny_, nz_;
-        float ngm;
-        if (vt + 1 < nvt)
-            slot_cols(vt + 1, nx_, ny_, nz_, ngm);
-        float *dst = f + fidx(vt, e, 0, lane, E, NP);
+    slot_cols(vt0, cx, cy, cz);
+    for (int vt = vt0; vt < vt1; vt++) {
+        int nx_ = 0, ny_ = 0, nz_ = 0;
+        if (vt + 1 < vt1)
+            slot_cols(vt + 1, nx_, ny_, nz_);
+        float *dst = f + ((int64_t)vt * npts + p0) * kWarp + lane;
 #pragma unroll 4
-        for (int i = w; i < NP; i += nw) {
+        for (int i = w; i < np; i += nw) {
             const float *t = tab + i * ntab;
-            __stcs(dst + i * kWarp, gm * (t[0] * t[cx] * t[cy] * t[cz]));
+            __stcs(dst + i * kWarp, t[cx] * t[cy] * t[cz]);
         }
-        if (vt + 1 < nvt) {
-            cx = nx_;
-            cy = ny_;
-            cz = nz_;
-            gm = ngm;
-        }
+        cx = nx_;
+        cy = ny_;
+        cz = nz_;
     }
 }
 
@@ -176,12 +193,24 @@ cudaError_t launch_init_maxwellian(float *f, const double *prim, const float *mi
                                    int nvt, int E, int NP, const int n[3], const double v0[3], const double dv[3],
                                    int *err, double *Q, double *warm, cudaStream_t s)
 {
-    const int smem = NP * (int)sizeof(double) + NP * (n[0] + n[1] + n[2] + 1) * (int)sizeof(float);
+    const int npts = E * NP, ntab = n[0] + n[1] + n[2] + 1;
+    // points per CTA: 64, so that two warps of them fill the lanes of the FP64 work, but 32 where that leaves
+    // fewer than two CTAs per SM, and no more than 96 KB of tables (two CTAs per SM) where the grid allows
+    const int per = 10 * (int)sizeof(double) + (ntab + 1) * (int)sizeof(float);
+    int PB = npts >= 64 * 304 ? 64 : 32;
+    PB = std::max(1, std::min(PB, 98304 / per));
+    const int smem = PB * per;
+    // runs of at least 32 tiles (their writing outweighs the tables that every run forms anew), as many as
+    // two CTAs per SM take
+    const int nb = (npts + PB - 1) / PB;
+    const int runs = std::max(1, std::min((nvt + 31) / 32, 304 / nb));
+    const int tiles = (nvt + runs - 1) / runs;
     cudaError_t e = cudaFuncSetAttribute(k_init_maxwellian, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess)
         return e;
-    k_init_maxwellian<<<E, 256, smem, s>>>(f, prim, mi, gmask, nslots, nvt, E, NP, n[0], n[1], n[2], v0[0], v0[1],
-                                           v0[2], dv[0], dv[1], dv[2], err, Q, warm);
+    k_init_maxwellian<<<dim3(nb, (nvt + tiles - 1) / tiles), 256, smem, s>>>(
+        f, prim, mi, gmask, nslots, nvt, npts, PB, tiles, n[0], n[1], n[2], v0[0], v0[1], v0[2], dv[0], dv[1], dv[2], err, Q,
+        warm);
     return cudaGetLastError();
 }
 
