@@ -668,6 +668,27 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
             atomicOr(A.err, kErrNewton);
         return;
     }
+    // the force's 1-D sums to m = 4 (FP64 throughout: with four lanes each forms its own axis's)
+    const bool force = A.force[0] != 0.0 || A.force[1] != 0.0 || A.force[2] != 0.0;
+    double Sf[3][5];
+    if (force) {
+        if constexpr (L == 1) {
+#pragma unroll
+            for (int d = 0; d < 3; d++)
+                sums64<5>(al[1 + d], -al[4], df_val(c0d[d]), df_val(hd[d]), A.n[d], A.dv[d], Sf[d]);
+        } else {
+            auto axis = [&](auto x, auto y, auto z) { return sub == 0 ? x : (sub == 1 ? y : z); };
+            const dfl c0 = axis(c0d[0], c0d[1], c0d[2]), h = axis(hd[0], hd[1], hd[2]);
+            double So[5];
+            sums64<5>(axis(al[1], al[2], al[3]), -al[4], df_val(c0), df_val(h), axis(A.n[0], A.n[1], A.n[2]),
+                      axis(A.dv[0], A.dv[1], A.dv[2]), So);
+#pragma unroll
+            for (int d = 0; d < 3; d++)
+#pragma unroll
+                for (int m = 0; m < 5; m++)
+                    Sf[d][m] = __shfl_sync(grp, So[m], d, 4);
+        }
+    }
     if (!writer)
         return;
 
@@ -726,13 +747,9 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
     // body force: source S = g (beta . psi~) with M[g psi~ psi~^T] beta = M[S psi~] =
     // (0, rho F / s, rho (U - V) . F / s^2), whose raw moments are (0, rho F, rho U . F); written as
     // the polynomial q0 + q . xi + q4 |xi|^2 in the raw velocity
-    if (A.force[0] != 0.0 || A.force[1] != 0.0 || A.force[2] != 0.0) {
-        double S[3][5];
-#pragma unroll
-        for (int d = 0; d < 3; d++)
-            sums64<5>(al[1 + d], -al[4], df_val(c0d[d]), df_val(hd[d]), A.n[d], A.dv[d], S[d]);
+    if (force) {
         double M[5], J[5][5], r[5], b[5];
-        assemble<double>(S, exp(al[0]), M, J);
+        assemble<double>(Sf, exp(al[0]), M, J);
         r[0] = 0.0;
         double uf = 0.0;
         for (int d = 0; d < 3; d++) {
