@@ -74,7 +74,8 @@ struct StageArgs {
     int n1;              // nodes per direction (p + 1)
     int vt0;             // first global tile of the chunk
     int nvt;             // tiles in the chunk
-    int G;               // tiles per warp task
+    int G;               // tiles per warp task and moment group
+    int T;               // tiles per CTA of k_stage3s (a multiple of G, set by its launch)
     int group0;          // global index of the chunk's first task group
     int nslots;          // total device velocity slots (= nvt_total * 32)
     int npts;            // n_x

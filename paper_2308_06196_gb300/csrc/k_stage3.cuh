@@ -689,7 +689,8 @@ cudaError_t launch3_any(const StageArgs &A, int mode, int oct, cudaStream_t s)
                         : (full ? launch3w_oct<N1, 1>(A, oct, s) : launch3w_oct<N1, 2>(A, oct, s));
     }
     else
-        return general ? launch3s_oct<N1, 1>(A, oct, s) : launch3s_oct<N1, 0>(A, oct, s);
+        return !general ? launch3s_oct<N1, 0>(A, oct, s)
+                        : (A.fpar ? launch3s_oct<N1, 2>(A, oct, s) : launch3s_oct<N1, 1>(A, oct, s));
 }
 
 }  // namespace bgk
