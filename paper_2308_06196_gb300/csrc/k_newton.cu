@@ -794,6 +794,8 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
 //                  point 512). Between 19,456 and 77,824 points 4 CTAs are faster alone (20,160 points 99
 //                  against 107) but slower where other work shares the SMs, since they hold twice the
 //                  registers: three contexts of 20,160 points stepped in turn 5.59 against 5.42 ms per pass.
+// With a body force the FP64 set-up that the four lanes repeat costs more than the latency it hides from
+// about 6,500 points on (9,720 points, three contexts in turn: 6.96 against 6.87 ms per pass).
 // The batched solve, whose arguments come from global memory, runs best at 4 CTAs.
 constexpr int kNewtonThreads = 128, kLanePoints = 152 * 4 * kNewtonThreads / 4;
 
@@ -839,7 +841,8 @@ cudaError_t launch_newton_batch(const NewtonArgs *d_args, const int *d_pt_start,
 
 cudaError_t launch_newton(const NewtonArgs &A, cudaStream_t s)
 {
-    if (A.npts <= kLanePoints)
+    const bool force = A.force[0] != 0.0 || A.force[1] != 0.0 || A.force[2] != 0.0;
+    if (A.npts <= (force ? kLanePoints / 3 : kLanePoints))
         k_newton<4, 4><<<newton_ctas(A.npts, 4), kNewtonThreads, 0, s>>>(A);
     else
         k_newton<1, 8><<<newton_ctas(A.npts, 1), kNewtonThreads, 0, s>>>(A);
