@@ -7,6 +7,7 @@
 //   stage 1: chunk c reads A[c]                      -> writes slot c
 //   stage 2: chunk c reads slot c (+ A[c])           -> writes slot c-1 (slot C for c = 0)
 //   stage 3: chunk c reads its stage-2 slot (+ A[c]) -> writes A[c] in place
+// (a small problem instead keeps two full stage buffers and launches all chunks of a stage together)
 // A stage reads neighbours only inside its own chunk, and chunks run in order on one stream, so a
 // slot is rewritten only after the launch that read it has finished. Memory = A + (C+1)/C arrays.
 #include <algorithm>
@@ -54,6 +55,9 @@ using namespace bgk;
 namespace {
 
 const double kPi = 3.14159265358979323846;
+// Stage buffers up to this size are kept in full (two f arrays instead of one and a chunk), so that the
+// chunks of a stage can go in one launch (see bgk_create)
+const int64_t kMergeBytes = 64ll << 20;
 const int kMinTuneG = 2;  // shortest task (tiles per warp task) the autotuner tries
 
 struct Chunk {
@@ -190,6 +194,7 @@ struct bgk_ctx {
     std::vector<unsigned char> toct_h;  // sign octant of every tile
     std::vector<Chunk> chunks;
     int64_t chunk_floats = 0;  // floats per pool slot
+    bool merged = false;       // small problem: one launch per stage over all chunks, two full stage buffers
     // device buffers
     float *fA = nullptr, *pool = nullptr;
     float *xi = nullptr, *mi = nullptr, *wpsi = nullptr, *gmask = nullptr, *ghost = nullptr;
@@ -313,6 +318,10 @@ StageArgs stage_args(bgk_ctx *c, const Chunk &ch)
     A.nvt = ch.nvt;
     A.G = c->G;
     A.group0 = ch.group0;
+    A.ngroups = ch.ngroups;
+    A.nseg = 1;
+    A.seg_vt[1] = ch.nvt;
+    A.seg_g[1] = ch.ngroups;
     A.nslots = c->nslots;
     A.npts = (int)c->npts;
     A.inv_tau = (float)(1.0 / c->tau);
@@ -329,6 +338,40 @@ StageArgs stage_args(bgk_ctx *c, const Chunk &ch)
     A.halo[1] = c->halo[1];
     A.eface = c->ne[1] * c->ne[2];
     return A;
+}
+
+// The launches of one stage: every chunk, or all chunks in one launch (the caller sets src, fn and dst).
+struct Launch {
+    StageArgs A;
+    int oct, vt0, chunk;  // octant (8: mixed), first tile, chunk index
+    int64_t real;         // velocities
+};
+
+std::vector<Launch> stage_launches(bgk_ctx *c)
+{
+    std::vector<Launch> L;
+    auto count = [&](int vt0, int nvt) {
+        int64_t n = 0;
+        for (int v = vt0 * kWarp; v < (vt0 + nvt) * kWarp; v++)
+            n += c->slotk[v] >= 0;
+        return n;
+    };
+    if (c->merged) {
+        const Chunk all{0, c->nvt, 0, c->ngroups, 8};
+        Launch l{stage_args(c, all), 8, 0, 0, count(0, c->nvt)};
+        l.A.nseg = (int)c->chunks.size();
+        for (int q = 0; q < l.A.nseg; q++) {
+            l.A.seg_vt[q + 1] = c->chunks[q].vt0 + c->chunks[q].nvt;
+            l.A.seg_g[q + 1] = c->chunks[q].group0 + c->chunks[q].ngroups;
+        }
+        L.push_back(l);
+        return L;
+    }
+    for (int q = 0; q < (int)c->chunks.size(); q++) {
+        const Chunk &ch = c->chunks[q];
+        L.push_back({stage_args(c, ch), ch.oct, ch.vt0, q, count(ch.vt0, ch.nvt)});
+    }
+    return L;
 }
 
 // Shu-Osher stage st (0, 1, 2) of step dt in FP32: b = 1, 1/4, 2/3 and an = 1 - b (exact), the
@@ -409,6 +452,17 @@ void ev_end(bgk_ctx *c)
 
 double *chunk_ptr64(bgk_ctx *c, double *base, int vt0) { return base + (int64_t)vt0 * c->E * c->NP * kWarp; }
 
+// Offset (in values) of chunk q's stage-1 (which = 0) or stage-2 (which = 1) output in the pool: the full
+// buffers of a small problem, or the rotating chunk slots -- stage 1 in slot q, stage 2 in slot q - 1
+// (slot C for chunk 0), which chunk q - 1 has read by then.
+int64_t pool_offset(const bgk_ctx *c, int q, int which)
+{
+    const int C = (int)c->chunks.size();
+    if (c->merged)
+        return ((int64_t)which * c->nvt + c->chunks[q].vt0) * c->E * c->NP * kWarp;
+    return (int64_t)(which == 0 ? q : (q == 0 ? C : q - 1)) * c->chunk_floats;
+}
+
 Moments64Args moments64_args(bgk_ctx *c)
 {
     Moments64Args M{};
@@ -456,10 +510,9 @@ int prologue(bgk_ctx *c, cudaStream_t s, bool have_q = false)
         CK(launch_newton(N, s));
         return BGK_OK;
     }
-    for (const Chunk &ch : c->chunks) {
-        StageArgs A = stage_args(c, ch);
-        A.src = chunk_ptr(c, c->fA, ch.vt0);
-        CK(launch_stage(A, c->p, 1, ch.oct, s));
+    for (Launch &l : stage_launches(c)) {
+        l.A.src = chunk_ptr(c, c->fA, l.vt0);
+        CK(launch_stage(l.A, c->p, 1, l.oct, s));
     }
     CK(launch_newton(newton_args(c, 1), s));
     return BGK_OK;
@@ -518,8 +571,7 @@ int enqueue_wall(bgk_ctx *c, const std::vector<const void *> &src, cudaStream_t 
 
 // One SSP-RK3 step of the plain all-FP64 form: per stage, the unfused stage kernel over every chunk,
 // the FP64 moments of all chunk outputs, then the Newton solve.
-int enqueue_step64(bgk_ctx *c, double dt, cudaStream_t s, const std::vector<int> &slot1,
-                   const std::vector<int> &slot2)
+int enqueue_step64(bgk_ctx *c, double dt, cudaStream_t s)
 {
     static const double an[3] = {0.0, 0.75, 1.0 / 3.0};
     static const double bb[3] = {1.0, 0.25, 2.0 / 3.0};
@@ -530,19 +582,17 @@ int enqueue_step64(bgk_ctx *c, double dt, cudaStream_t s, const std::vector<int>
             std::vector<const void *> srcs(C);
             for (int q = 0; q < C; q++) {
                 double *Aq = chunk_ptr64(c, c->fA64, c->chunks[q].vt0);
-                srcs[q] = st == 0 ? (const void *)Aq
-                                  : (const void *)(c->pool64 + (int64_t)(st == 1 ? slot1[q] : slot2[q]) * c->chunk_floats);
+                srcs[q] = st == 0 ? (const void *)Aq : (const void *)(c->pool64 + pool_offset(c, q, st - 1));
             }
             int rc = enqueue_wall(c, srcs, s);
             if (rc)
                 return rc;
         }
         CK(launch_table64(c->etab64, c->par64, table64_args(c), (int)c->npts, s));
-        for (int q = 0; q < C; q++) {
-            const Chunk &ch = c->chunks[q];
-            double *Aq = chunk_ptr64(c, c->fA64, ch.vt0);
-            double *s1 = c->pool64 + (int64_t)slot1[q] * c->chunk_floats;
-            double *s2 = c->pool64 + (int64_t)slot2[q] * c->chunk_floats;
+        for (const Launch &l : stage_launches(c)) {
+            double *Aq = chunk_ptr64(c, c->fA64, l.vt0);
+            double *s1 = c->pool64 + pool_offset(c, l.chunk, 0);
+            double *s2 = c->pool64 + pool_offset(c, l.chunk, 1);
             Stage64Args A{};
             A.src = st == 0 ? Aq : (st == 1 ? s1 : s2);
             A.fn = st == 0 ? nullptr : Aq;
@@ -562,8 +612,8 @@ int enqueue_step64(bgk_ctx *c, double dt, cudaStream_t s, const std::vector<int>
                 A.h[d] = c->h[d];
             A.N1 = c->N1;
             A.NP = c->NP;
-            A.vt0 = ch.vt0;
-            A.nvt = ch.nvt;
+            A.vt0 = l.A.vt0;
+            A.nvt = l.A.nvt;
             A.nslots = c->nslots;
             A.an = an[st];
             A.b = bb[st];
@@ -576,15 +626,15 @@ int enqueue_step64(bgk_ctx *c, double dt, cudaStream_t s, const std::vector<int>
             A.ftab = c->ftab;
             A.fbase = c->fbase;
             A.rhowu = c->rhowu64;
-            int64_t real = 0;
-            for (int v = ch.vt0 * kWarp; v < (ch.vt0 + ch.nvt) * kWarp; v++)
-                real += c->slotk[v] >= 0;
-            ev_begin(c, 0, (double)real * c->npts * sizeof(double) * (st == 0 ? 2 : 3));
+            ev_begin(c, 0, (double)l.real * c->npts * sizeof(double) * (st == 0 ? 2 : 3));
             CK(launch_stage64(A, s));
             if (c->opts.limiter)
-                CK(launch_limit64(A.dst, ch.nvt, c->E, c->NP, c->N1, c->dim, c->ops64, c->ijac64, s));
+                CK(launch_limit64(A.dst, A.nvt, c->E, c->NP, c->N1, c->dim, c->ops64, c->ijac64, s));
             ev_end(c);
-            M.base[q] = A.dst;
+        }
+        for (int q = 0; q < C; q++) {
+            const Chunk &ch = c->chunks[q];
+            M.base[q] = st == 2 ? chunk_ptr64(c, c->fA64, ch.vt0) : c->pool64 + pool_offset(c, q, st);
             M.vt0[q] = ch.vt0;
             M.nvt[q] = ch.nvt;
         }
@@ -601,14 +651,8 @@ int enqueue_stage(bgk_ctx *c, double dt, int st, cudaStream_t s);
 // One SSP-RK3 step: three stages, each over all chunks, each followed by the Newton solve.
 int enqueue_step(bgk_ctx *c, double dt, cudaStream_t s)
 {
-    const int C = (int)c->chunks.size();
-    std::vector<int> slot1(C), slot2(C);
-    for (int q = 0; q < C; q++) {
-        slot1[q] = q;
-        slot2[q] = q == 0 ? C : q - 1;
-    }
     if (c->prec == BGK_FP64)
-        return enqueue_step64(c, dt, s, slot1, slot2);
+        return enqueue_step64(c, dt, s);
     for (int st = 0; st < 3; st++) {
         int rc = enqueue_stage(c, dt, st, s);
         if (rc)
@@ -617,79 +661,38 @@ int enqueue_step(bgk_ctx *c, double dt, cudaStream_t s)
     return BGK_OK;
 }
 
-// Pool slots of the FP32-split stage outputs: chunk q's stage-1 output in slot q, its stage-2 output in
-// slot q - 1 (slot C for chunk 0), which chunk q - 1 has read by then.
-void stage_slots(const bgk_ctx *c, std::vector<int> &slot1, std::vector<int> &slot2)
-{
-    const int C = (int)c->chunks.size();
-    slot1.resize(C);
-    slot2.resize(C);
-    for (int q = 0; q < C; q++) {
-        slot1[q] = q;
-        slot2[q] = q == 0 ? C : q - 1;
-    }
-}
-
 // The source of stage st (0, 1, 2) of chunk q (FP32-split form): f^n, the stage-1 or the stage-2 output.
 float *stage_source(bgk_ctx *c, int q, int st)
 {
-    std::vector<int> slot1, slot2;
-    stage_slots(c, slot1, slot2);
-    if (st == 0)
-        return chunk_ptr(c, c->fA, c->chunks[q].vt0);
-    return c->pool + (int64_t)(st == 1 ? slot1[q] : slot2[q]) * c->chunk_floats;
+    return st == 0 ? chunk_ptr(c, c->fA, c->chunks[q].vt0) : c->pool + pool_offset(c, q, st - 1);
 }
 
 // Stage st of one SSP-RK3 step of the FP32-split form: the wall densities of the stage source, the stage
 // kernel over every chunk, the Newton solve of the stage output.
 int enqueue_stage(bgk_ctx *c, double dt, int st, cudaStream_t s)
 {
-    const int C = (int)c->chunks.size();
-    std::vector<int> slot1, slot2;
-    stage_slots(c, slot1, slot2);
-    {
-        if (c->has_wall) {
-            std::vector<const void *> srcs(C);
-            for (int q = 0; q < C; q++) {
-                float *Aq = chunk_ptr(c, c->fA, c->chunks[q].vt0);
-                srcs[q] = st == 0 ? (const void *)Aq
-                                  : (const void *)(c->pool + (int64_t)(st == 1 ? slot1[q] : slot2[q]) * c->chunk_floats);
-            }
-            int rc = enqueue_wall(c, srcs, s);
-            if (rc)
-                return rc;
-        }
-        for (int q = 0; q < C; q++) {
-            const Chunk &ch = c->chunks[q];
-            StageArgs A = stage_args(c, ch);
-            float *Aq = chunk_ptr(c, c->fA, ch.vt0);
-            float *s1 = c->pool + (int64_t)slot1[q] * c->chunk_floats;
-            float *s2 = c->pool + (int64_t)slot2[q] * c->chunk_floats;
-            if (st == 0) {
-                A.src = Aq;
-                A.fn = nullptr;
-                A.dst = s1;
-            } else if (st == 1) {
-                A.src = s1;
-                A.fn = Aq;
-                A.dst = s2;
-            } else {
-                A.src = s2;
-                A.fn = Aq;
-                A.dst = Aq;
-            }
-            stage_coeffs(A, st, dt, c->tau);
-            int64_t real = 0;
-            for (int v = ch.vt0 * kWarp; v < (ch.vt0 + ch.nvt) * kWarp; v++)
-                real += c->slotk[v] >= 0;
-            ev_begin(c, 0, (double)real * c->npts * sizeof(float) * (st == 0 ? 2 : 3));
-            CK(launch_stage(A, c->p, 0, ch.oct, s));
-            ev_end(c);
-        }
-        ev_begin(c, 1, 0.0);
-        CK(launch_newton(newton_args(c, 0), s));
+    if (c->has_wall) {
+        std::vector<const void *> srcs(c->chunks.size());
+        for (size_t q = 0; q < srcs.size(); q++)
+            srcs[q] = stage_source(c, (int)q, st);
+        int rc = enqueue_wall(c, srcs, s);
+        if (rc)
+            return rc;
+    }
+    for (Launch &l : stage_launches(c)) {
+        StageArgs &A = l.A;
+        float *Aq = chunk_ptr(c, c->fA, l.vt0);
+        A.src = stage_source(c, l.chunk, st);
+        A.fn = st == 0 ? nullptr : Aq;
+        A.dst = st == 2 ? Aq : stage_source(c, l.chunk, st + 1);
+        stage_coeffs(A, st, dt, c->tau);
+        ev_begin(c, 0, (double)l.real * c->npts * sizeof(float) * (st == 0 ? 2 : 3));
+        CK(launch_stage(A, c->p, 0, l.oct, s));
         ev_end(c);
     }
+    ev_begin(c, 1, 0.0);
+    CK(launch_newton(newton_args(c, 0), s));
+    ev_end(c);
     return BGK_OK;
 }
 
@@ -938,9 +941,15 @@ int bgk_create(const bgk_mesh *mesh, int p, const bgk_vgrid *vg, double tau, con
     for (int q = 0; q < 6; q++)
         c->mesh.bc[q] = c->bc[q];
 
-    // memory check before any allocation
+    // Small problems: all chunks of a stage in one launch. A stage of a few microseconds per chunk is bound by
+    // the launches and by their nearly empty chip (a 24-element shock tube, 12^3 velocities, 20 steps with a
+    // checkpoint: 3.42 -> 1.80 ms; 3 x 2 x 4 elements at p = 3, 14^3 velocities, 17 MB of f: 0.43 -> 0.34 ms
+    // per pass); above the limit the octants' own kernels and the smaller memory win.
     const int64_t fA = (int64_t)c->nvt * E * c->NP * kWarp;
-    const int64_t need = (fA + (int64_t)(c->chunks.size() + 1) * c->chunk_floats) * c->esize +
+    c->merged = c->opts.chunks == 0 && c->chunks.size() > 1 && fA * c->esize <= kMergeBytes;
+    const int64_t pool = c->merged ? 2 * fA : (int64_t)(c->chunks.size() + 1) * c->chunk_floats;
+    // memory check before any allocation
+    const int64_t need = (fA + pool) * c->esize +
                          (int64_t)c->max_groups * 5 * c->npts * 4 + c->npts * (5 * 8 * 3 + kParamStride * 4) +
                          (int64_t)c->nslots * 4 * 25 +
                          (c->prec == BGK_FP64 ? c->npts * 8 * (c->nv[0] + c->nv[1] + c->nv[2]) : 0) +
@@ -960,7 +969,7 @@ int bgk_create(const bgk_mesh *mesh, int p, const bgk_vgrid *vg, double tau, con
         return bail(BGK_ENOMEM, std::string("cudaMalloc failed: ") + #ptr);
     if (c->prec == BGK_FP64) {
         AL(c->fA64, fA);
-        AL(c->pool64, (c->chunks.size() + 1) * c->chunk_floats);
+        AL(c->pool64, pool);
         AL(c->xi64, 3 * c->nslots);
         AL(c->wpsi64, 5 * c->nslots);
         AL(c->ghost64, 6 * c->nslots);
@@ -970,7 +979,7 @@ int bgk_create(const bgk_mesh *mesh, int p, const bgk_vgrid *vg, double tau, con
             AL(c->itau64, c->npts);
     } else {
         AL(c->fA, fA);
-        AL(c->pool, (c->chunks.size() + 1) * c->chunk_floats);
+        AL(c->pool, pool);
     }
     AL(c->xi, 3 * c->nslots);
     AL(c->mi, 3 * c->nslots);
@@ -1792,23 +1801,18 @@ int bgk_autotune(bgk_ctx *c, int *g_out)
     CK(cudaEventCreate(&e1));
     float best = 1e30f;
     int bestG = c->G;
-    const int C = (int)c->chunks.size();
     for (int G : task_length_candidates(maxc)) {
         set_task_length(c, G);
         float tot = 0.f;
         for (int rep = 0; rep < 3; rep++) {
             CK(cudaEventRecord(e0, c->stream));
-            // stage 2 of every chunk: reads the first pool slots and f^n, writes the second slots
-            for (int q = 0; q < C; q++) {
-                const Chunk &ch = c->chunks[q];
-                StageArgs A = stage_args(c, ch);
-                A.src = c->pool + (int64_t)q * c->chunk_floats;
-                A.fn = chunk_ptr(c, c->fA, ch.vt0);
-                A.dst = c->pool + (int64_t)(q == 0 ? C : q - 1) * c->chunk_floats;
-                stage_coeffs(A, 1, 0.1 * c->tau, c->tau);
-                if (q == 0 && C > 1)
-                    A.dst = c->pool + (int64_t)C * c->chunk_floats;
-                CK(launch_stage(A, c->p, 0, ch.oct, c->stream));
+            // stage 2 of every chunk: reads the stage-1 outputs and f^n, writes the stage-2 outputs
+            for (Launch &l : stage_launches(c)) {
+                l.A.src = stage_source(c, l.chunk, 1);
+                l.A.fn = chunk_ptr(c, c->fA, l.vt0);
+                l.A.dst = stage_source(c, l.chunk, 2);
+                stage_coeffs(l.A, 1, 0.1 * c->tau, c->tau);
+                CK(launch_stage(l.A, c->p, 0, l.oct, c->stream));
             }
             CK(cudaEventRecord(e1, c->stream));
             CK(cudaEventSynchronize(e1));

@@ -76,7 +76,11 @@ struct StageArgs {
     int nvt;             // tiles in the chunk
     int G;               // tiles per warp task and moment group
     int T;               // tiles per CTA of k_stage3s (a multiple of G, set by its launch)
-    int group0;          // global index of the chunk's first task group
+    int group0;          // global index of the launch's first task group
+    int ngroups;         // task groups of the launch
+    // the velocity chunks of the launch (one, or all of them in a small problem's launch): chunk s holds local
+    // tiles seg_vt[s] .. seg_vt[s+1] - 1 in groups seg_g[s] .. seg_g[s+1] - 1 (task_tiles)
+    int nseg, seg_vt[10], seg_g[10];
     int nslots;          // total device velocity slots (= nvt_total * 32)
     int npts;            // n_x
     float an, b;         // Shu-Osher coefficients: out = an f^n + b (f_s + dt L(f_s))

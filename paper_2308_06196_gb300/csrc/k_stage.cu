@@ -81,8 +81,8 @@ __device__ __forceinline__ void line_task(const StageArgs &A, const int task, co
     const int eb = (task % nEB) * K;
     const int ne = min(K, E - eb);
     const int nr = ne * N1;  // real rows of the run
-    const int vl0 = gl * A.G;
-    const int vl1 = min(vl0 + A.G, A.nvt);
+    int vl0, vl1;
+    task_tiles(A, gl, vl0, vl1);
     int ec[3] = {eb, 0, 0};
     const int enL = upwind_neighbour(A.mesh, ec, 0, true);  // outside neighbours of the run
     ec[0] = eb + ne - 1;
@@ -320,7 +320,7 @@ template <int N1>
 __host__ __device__ int line_tasks(const StageArgs &A)
 {
     constexpr int K = line_run<N1>();
-    return ((A.mesh.nelem + K - 1) / K) * ((A.nvt + A.G - 1) / A.G);
+    return ((A.mesh.nelem + K - 1) / K) * A.ngroups;
 }
 
 int stage1d_tasks(const StageArgs &A)

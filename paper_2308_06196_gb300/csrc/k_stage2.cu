@@ -41,8 +41,8 @@ __global__ void __launch_bounds__(kWarp *kWarpsPerCta, BGK_STAGE2_MINCTAS) k_sta
     if (e >= E)
         return;  // the warps of a CTA never wait for one another
     QuadSmem<N1> &sm = smw[w];
-    const int vl0 = gl * A.G;
-    const int vl1 = min(vl0 + A.G, A.nvt);
+    int vl0, vl1;
+    task_tiles(A, gl, vl0, vl1);
     const int ec[3] = {e % A.mesh.ne[0], e / A.mesh.ne[0], 0};
 
     if (MODE == 0) {
@@ -373,9 +373,8 @@ __global__ void __launch_bounds__(kWarp *kWarpsPerCta, BGK_STAGE2_MINCTAS) k_sta
 template <int N1, int MODE, int OCT>
 cudaError_t launch2(const StageArgs &A, cudaStream_t s)
 {
-    const int ngroups = (A.nvt + A.G - 1) / A.G;
     const int EB = (A.mesh.nelem + kWarpsPerCta - 1) / kWarpsPerCta;
-    k_stage2<N1, MODE, OCT><<<EB * ngroups, kWarp * kWarpsPerCta, 0, s>>>(A);
+    k_stage2<N1, MODE, OCT><<<EB * A.ngroups, kWarp * kWarpsPerCta, 0, s>>>(A);
     return cudaGetLastError();
 }
 

@@ -124,8 +124,8 @@ __global__ void __launch_bounds__(kWarp *N1, (N1 >= 4 ? (GEN || CURV ? BGK_STAGE
     const int E = A.mesh.nelem;
     const int gl = blockIdx.x / E;
     const int e = blockIdx.x % E;
-    const int vl0 = gl * A.G;
-    const int vl1 = min(vl0 + A.G, A.nvt);
+    int vl0, vl1;
+    task_tiles(A, gl, vl0, vl1);
     int ec[3];
     ec[0] = e % A.mesh.ne[0];
     ec[1] = (e / A.mesh.ne[0]) % A.mesh.ne[1];
@@ -636,9 +636,8 @@ __global__ void __launch_bounds__(kWarp *N1, (N1 >= 4 ? (GEN || CURV ? BGK_STAGE
 template <int N1, int MODE, int OCT, int GEN, int CURV = 0>
 cudaError_t launch3(const StageArgs &A, cudaStream_t s)
 {
-    const int ngroups = (A.nvt + A.G - 1) / A.G;
     k_stage3<N1, MODE, OCT, GEN, CURV>
-        <<<A.mesh.nelem * ngroups, kWarp * N1, stage3_smem_bytes<N1, GEN, CURV>(), s>>>(A);
+        <<<A.mesh.nelem * A.ngroups, kWarp * N1, stage3_smem_bytes<N1, GEN, CURV>(), s>>>(A);
     return cudaGetLastError();
 }
 

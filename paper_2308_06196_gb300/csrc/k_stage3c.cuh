@@ -99,8 +99,8 @@ __global__ void __launch_bounds__(kWarp *N1, (N1 >= 4 ? BGK_STAGE3C_MINCTAS_P3 :
     const int E = A.mesh.nelem;
     const int gl = blockIdx.x / E;
     const int e = blockIdx.x % E;
-    const int vl0 = gl * A.G;
-    const int vl1 = min(vl0 + A.G, A.nvt);
+    int vl0, vl1;
+    task_tiles(A, gl, vl0, vl1);
     int ec[3];
     ec[0] = e % A.mesh.ne[0];
     ec[1] = (e / A.mesh.ne[0]) % A.mesh.ne[1];
@@ -710,8 +710,7 @@ cudaError_t prepare3c()
 template <int N1, int GEN>
 cudaError_t launch3c(const StageArgs &A, cudaStream_t s)
 {
-    const int ngroups = (A.nvt + A.G - 1) / A.G;
-    k_stage3c<N1, GEN><<<A.mesh.nelem * ngroups, kWarp * N1, sizeof(Stage3cSmem<N1, GEN>), s>>>(A);
+    k_stage3c<N1, GEN><<<A.mesh.nelem * A.ngroups, kWarp * N1, sizeof(Stage3cSmem<N1, GEN>), s>>>(A);
     return cudaGetLastError();
 }
 

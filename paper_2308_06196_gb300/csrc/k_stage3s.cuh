@@ -86,8 +86,14 @@ __global__ void __launch_bounds__(kWarp *N1 / 2, kStage3sCtas<GEN>)
     const int lz = 2 * w + hf;                       // this lane's z-layer (and z-line slice iy)
     const int E = A.mesh.nelem;
     const int e = blockIdx.x % E;
-    const int vl0 = (blockIdx.x / E) * A.T;
-    const int vl1 = min(vl0 + A.T, A.nvt);
+    int vl0, vl1, g0 = blockIdx.x / E;  // tiles, first moment group
+    if (A.T == A.G) {
+        task_tiles(A, g0, vl0, vl1);
+    } else {  // several groups of the launch's one chunk
+        vl0 = g0 * A.T;
+        vl1 = min(vl0 + A.T, A.nvt);
+        g0 = vl0 / A.G;
+    }
     int ec[3];
     ec[0] = e % A.mesh.ne[0];
     ec[1] = (e / A.mesh.ne[0]) % A.mesh.ne[1];
@@ -524,8 +530,8 @@ __global__ void __launch_bounds__(kWarp *N1 / 2, kStage3sCtas<GEN>)
             fence_proxy_async();
             issue(ys, vl + 1, bF);
         }
-        if (!more || (vl + 1) % A.G == 0) {  // the end of a moment group: combine the 4 velocity eighths of a row
-            const int grp = A.group0 + vl / A.G;
+        if (!more || (vl + 1 - vl0) % A.G == 0) {  // the end of a moment group: combine the 4 velocity eighths of a row
+            const int grp = A.group0 + g0 + (vl - vl0) / A.G;
 #pragma unroll
             for (int r = 0; r < NR; r++)
 #pragma unroll
@@ -562,9 +568,9 @@ cudaError_t launch3s(const StageArgs &A0, cudaStream_t s)
     StageArgs A = A0;
     const int64_t E = A.mesh.nelem;
     A.T = A.G;
-    while (A.T < A.nvt && E * ((A.nvt + 2 * A.T - 1) / (2 * A.T)) >= 8 * kWave)
+    while (A.nseg == 1 && A.T < A.nvt && E * ((A.nvt + 2 * A.T - 1) / (2 * A.T)) >= 8 * kWave)
         A.T *= 2;
-    k_stage3s<N1, OCT, GEN><<<A.mesh.nelem * ((A.nvt + A.T - 1) / A.T), kWarp * N1 / 2, sizeof(Stage3sSmem<N1, GEN>), s>>>(A);
+    k_stage3s<N1, OCT, GEN><<<A.mesh.nelem * (A.T == A.G ? A.ngroups : (A.nvt + A.T - 1) / A.T), kWarp * N1 / 2, sizeof(Stage3sSmem<N1, GEN>), s>>>(A);
     return cudaGetLastError();
 }
 

@@ -66,8 +66,8 @@ __global__ void __launch_bounds__(kWarp *BGK_STAGE3W_WARPS, (N1 == 3 ? BGK_STAGE
     const int e = (blockIdx.x % nblk) * BGK_STAGE3W_WARPS + wq;
     if (e >= E)  // no barrier below involves other warps
         return;
-    const int vl0 = gl * A.G;
-    const int vl1 = min(vl0 + A.G, A.nvt);
+    int vl0, vl1;
+    task_tiles(A, gl, vl0, vl1);
     int ec[3];
     ec[0] = e % A.mesh.ne[0];
     ec[1] = (e / A.mesh.ne[0]) % A.mesh.ne[1];
@@ -272,12 +272,11 @@ __global__ void __launch_bounds__(kWarp *BGK_STAGE3W_WARPS, (N1 == 3 ? BGK_STAGE
                 fl[j] = f[j + N1 * ln];
                 v[j] = sm.sl[kx][j + N1 * ln][lane];
             }
-            const float bx = gx * rw[ln];
             if (l0) {
-                const float tj = trace_jump<N1, true>(v, fl[0], A.ops), gj = bx - fl[0];
+                const float tj = trace_jump<N1, true>(v, fl[0], A.ops), gj = fmaf(gx, rw[ln], -fl[0]);
                 line_sums_jump<N1, true>(sv, fl, inx ? tj : gj, A.ops);
             } else {
-                const float tj = trace_jump<N1, false>(v, fl[N1 - 1], A.ops), gj = bx - fl[N1 - 1];
+                const float tj = trace_jump<N1, false>(v, fl[N1 - 1], A.ops), gj = fmaf(gx, rw[ln], -fl[N1 - 1]);
                 line_sums_jump<N1, false>(sv, fl, inx ? tj : gj, A.ops);
             }
 #pragma unroll
@@ -297,12 +296,11 @@ __global__ void __launch_bounds__(kWarp *BGK_STAGE3W_WARPS, (N1 == 3 ? BGK_STAGE
                     fl[j] = f[ix + N1 * j + NQ * iz];
                     v[j] = sm.sl[ky][ix + N1 * j + NQ * iz][lane];
                 }
-                const float by = gy * rw[ix + N1 * iz];
                 if (l1) {
-                    const float tj = trace_jump<N1, true>(v, fl[0], A.ops), gj = by - fl[0];
+                    const float tj = trace_jump<N1, true>(v, fl[0], A.ops), gj = fmaf(gy, rw[ix + N1 * iz], -fl[0]);
                     line_sums_jump<N1, true>(sv, fl, iny ? tj : gj, A.ops);
                 } else {
-                    const float tj = trace_jump<N1, false>(v, fl[N1 - 1], A.ops), gj = by - fl[N1 - 1];
+                    const float tj = trace_jump<N1, false>(v, fl[N1 - 1], A.ops), gj = fmaf(gy, rw[ix + N1 * iz], -fl[N1 - 1]);
                     line_sums_jump<N1, false>(sv, fl, iny ? tj : gj, A.ops);
                 }
 #pragma unroll
@@ -327,12 +325,11 @@ __global__ void __launch_bounds__(kWarp *BGK_STAGE3W_WARPS, (N1 == 3 ? BGK_STAGE
                 fl[j] = f[q + NQ * j];
                 v[j] = sm.sl[ka][q + NQ * j][lane];
             }
-            const float bz = gz * rw[q];
             if (l2) {
-                const float tj = trace_jump<N1, true>(v, fl[0], A.ops), gj = bz - fl[0];
+                const float tj = trace_jump<N1, true>(v, fl[0], A.ops), gj = fmaf(gz, rw[q], -fl[0]);
                 line_sums_jump<N1, true>(sv, fl, inz ? tj : gj, A.ops);
             } else {
-                const float tj = trace_jump<N1, false>(v, fl[N1 - 1], A.ops), gj = bz - fl[N1 - 1];
+                const float tj = trace_jump<N1, false>(v, fl[N1 - 1], A.ops), gj = fmaf(gz, rw[q], -fl[N1 - 1]);
                 line_sums_jump<N1, false>(sv, fl, inz ? tj : gj, A.ops);
             }
 #pragma unroll
@@ -494,9 +491,8 @@ __global__ void __launch_bounds__(kWarp *BGK_STAGE3W_WARPS, (N1 == 3 ? BGK_STAGE
 template <int N1, int OCT, int GEN>
 cudaError_t launch3w(const StageArgs &A, cudaStream_t s)
 {
-    const int ngroups = (A.nvt + A.G - 1) / A.G;
     const int nblk = (A.mesh.nelem + BGK_STAGE3W_WARPS - 1) / BGK_STAGE3W_WARPS;
-    k_stage3w<N1, OCT, GEN><<<nblk * ngroups, kWarp * BGK_STAGE3W_WARPS,
+    k_stage3w<N1, OCT, GEN><<<nblk * A.ngroups, kWarp * BGK_STAGE3W_WARPS,
                               BGK_STAGE3W_WARPS * sizeof(Stage3wWarp<N1, GEN>), s>>>(A);
     return cudaGetLastError();
 }

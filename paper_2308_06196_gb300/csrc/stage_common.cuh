@@ -4,6 +4,17 @@
 
 namespace bgk {
 
+// Tiles [vl0, vl1) of task group gl of a launch: groups of G tiles that do not cross a chunk's end, so the
+// partial moment sums are the same whether the chunks are launched one by one or together.
+__device__ __forceinline__ void task_tiles(const StageArgs &A, int gl, int &vl0, int &vl1)
+{
+    int s = 0;
+    while (s + 1 < A.nseg && gl >= A.seg_g[s + 1])
+        s++;
+    vl0 = A.seg_vt[s] + (gl - A.seg_g[s]) * A.G;
+    vl1 = min(vl0 + A.G, A.seg_vt[s + 1]);
+}
+
 // fused multiply-add on two packed FP32 lanes (sm_100+): d = a * b + c, element-wise
 __device__ __forceinline__ unsigned long long ffma2(unsigned long long a, unsigned long long b,
                                                     unsigned long long c)
