@@ -786,18 +786,20 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
 
 // The two forms of the solve, by the number of points (128-thread CTAs on 152 SMs; us per launch alone,
 // before -> now, with the partial sums' loads four groups at a time):
-//   up to 19,456   one wave of latency: four lanes share a point, 4 CTAs per SM leave the 128 registers that
-//                  avoid spills (72 points 44 -> 23; 6,000 points 80 -> 39; 12,000 points 90 -> 47);
+//   up to 9,728    latency: four lanes share a point, 4 CTAs per SM leave the 128 registers that avoid
+//                  spills (72 points 44 -> 23; 6,000 points 80 -> 39). Up to 19,456 points (one wave) the launch
+//                  itself is still shorter (12,000 points 90 -> 47), but the FP64 set-up that the four lanes
+//                  repeat costs other work on the SMs more (13,440 points, three contexts in turn 5.57
+//                  against 5.49 ms per pass);
 //   beyond         the FP64 pipe (a warp instruction per 16 clocks and SM; some 230 per point in the set-up
 //                  and the outputs) and the chains' latency: a thread per point, 8 CTAs (64 registers,
 //                  spilling to L1) keep it busiest (262,144 points 170 -> 164; 4 CTAs 198, four lanes per
-//                  point 512). Between 19,456 and 77,824 points 4 CTAs are faster alone (20,160 points 99
-//                  against 107) but slower where other work shares the SMs, since they hold twice the
-//                  registers: three contexts of 20,160 points stepped in turn 5.59 against 5.42 ms per pass.
-// With a body force the FP64 set-up that the four lanes repeat costs more than the latency it hides from
-// about 6,500 points on (9,720 points, three contexts in turn: 6.96 against 6.87 ms per pass).
+//                  point 512; 20,160 points 99 alone with 4 CTAs against 107, but three contexts in turn 5.59
+//                  against 5.42 ms per pass).
+// With a body force the set-up is longer and the limit two thirds of that (9,720 points, three contexts in turn:
+// 6.96 against 6.87 ms per pass).
 // The batched solve, whose arguments come from global memory, runs best at 4 CTAs.
-constexpr int kNewtonThreads = 128, kLanePoints = 152 * 4 * kNewtonThreads / 4;
+constexpr int kNewtonThreads = 128, kLanePoints = 152 * 2 * kNewtonThreads / 4;
 
 template <int L, int MINCTAS>
 __global__ void __launch_bounds__(kNewtonThreads, MINCTAS) k_newton(const NewtonArgs A)
@@ -842,7 +844,7 @@ cudaError_t launch_newton_batch(const NewtonArgs *d_args, const int *d_pt_start,
 cudaError_t launch_newton(const NewtonArgs &A, cudaStream_t s)
 {
     const bool force = A.force[0] != 0.0 || A.force[1] != 0.0 || A.force[2] != 0.0;
-    if (A.npts <= (force ? kLanePoints / 3 : kLanePoints))
+    if (A.npts <= (force ? kLanePoints * 2 / 3 : kLanePoints))
         k_newton<4, 4><<<newton_ctas(A.npts, 4), kNewtonThreads, 0, s>>>(A);
     else
         k_newton<1, 8><<<newton_ctas(A.npts, 1), kNewtonThreads, 0, s>>>(A);

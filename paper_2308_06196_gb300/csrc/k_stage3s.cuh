@@ -555,8 +555,18 @@ __global__ void __launch_bounds__(kWarp *N1 / 2, kStage3sCtas<GEN>)
     }
 }
 
-// Tiles per CTA: as many whole moment groups as leave eight waves of CTAs (a CTA's first copies are not hidden
-// behind its own work: 16^3 elements, 54 tiles per octant, ran 3 % faster with 32 tiles per CTA than with 8).
+// Tiles per CTA (A.T): as many whole moment groups as leave eight waves of `wave` CTAs (a CTA's first copies are
+// not hidden behind its own work: 16^3 elements, 54 tiles per octant, ran 3 % faster with 32 tiles per CTA
+// than with 8). Returns the CTAs per element.
+inline int stage3_tasks(StageArgs &A, int wave)
+{
+    const int64_t E = A.mesh.nelem;
+    A.T = A.G;
+    while (A.nseg == 1 && A.T < A.nvt && E * ((A.nvt + 2 * A.T - 1) / (2 * A.T)) >= 8 * wave)
+        A.T *= 2;
+    return A.T == A.G ? A.ngroups : (A.nvt + A.T - 1) / A.T;
+}
+
 template <int N1, int OCT, int GEN>
 cudaError_t launch3s(const StageArgs &A0, cudaStream_t s)
 {
@@ -564,13 +574,9 @@ cudaError_t launch3s(const StageArgs &A0, cudaStream_t s)
     static_assert(offsetof(Sm, tab) % 16 == 0 && offsetof(Sm, par) % 16 == 0 && offsetof(Sm, fpar) % 16 == 0 &&
                       offsetof(Sm, lim) % 16 == 0 && offsetof(Sm, bar) % 8 == 0,
                   "8- and 16-byte shared accesses");
-    constexpr int kWave = 152 * kStage3sCtas<GEN>;
     StageArgs A = A0;
-    const int64_t E = A.mesh.nelem;
-    A.T = A.G;
-    while (A.nseg == 1 && A.T < A.nvt && E * ((A.nvt + 2 * A.T - 1) / (2 * A.T)) >= 8 * kWave)
-        A.T *= 2;
-    k_stage3s<N1, OCT, GEN><<<A.mesh.nelem * (A.T == A.G ? A.ngroups : (A.nvt + A.T - 1) / A.T), kWarp * N1 / 2, sizeof(Stage3sSmem<N1, GEN>), s>>>(A);
+    const int ctas = stage3_tasks(A, 152 * kStage3sCtas<GEN>);
+    k_stage3s<N1, OCT, GEN><<<A.mesh.nelem * ctas, kWarp * N1 / 2, sizeof(Sm), s>>>(A);
     return cudaGetLastError();
 }
 

@@ -8,6 +8,11 @@ namespace bgk {
 // partial moment sums are the same whether the chunks are launched one by one or together.
 __device__ __forceinline__ void task_tiles(const StageArgs &A, int gl, int &vl0, int &vl1)
 {
+    if (A.nseg == 1) {  // (the usual launch: no search, which a short task would feel)
+        vl0 = gl * A.G;
+        vl1 = min(vl0 + A.G, A.nvt);
+        return;
+    }
     int s = 0;
     while (s + 1 < A.nseg && gl >= A.seg_g[s + 1])
         s++;
