@@ -58,6 +58,11 @@ const double kPi = 3.14159265358979323846;
 // Stage buffers up to this size are kept in full (two f arrays instead of one and a chunk), so that the
 // chunks of a stage can go in one launch (see bgk_create)
 const int64_t kMergeBytes = 64ll << 20;
+// Tiles per task of the batched line launches (whole moment groups of at least this, see batch_upload)
+#ifndef BGK_BATCH_TILES
+#define BGK_BATCH_TILES 16
+#endif
+const int kBatchTiles = BGK_BATCH_TILES;
 const int kMinTuneG = 2;  // shortest task (tiles per warp task) the autotuner tries
 
 struct Chunk {
@@ -318,7 +323,8 @@ StageArgs stage_args(bgk_ctx *c, const Chunk &ch)
     A.nvt = ch.nvt;
     A.G = c->G;
     A.group0 = ch.group0;
-    A.ngroups = ch.ngroups;
+    A.ngroups = A.ntasks = ch.ngroups;
+    A.R = 1;
     A.nseg = 1;
     A.seg_vt[1] = ch.nvt;
     A.seg_g[1] = ch.ngroups;
@@ -1942,6 +1948,8 @@ int batch_upload(bgk_batch *b, const double *dt)
             real += c->slotk[v] >= 0;
         for (int st = 0; st < 3; st++) {
             StageArgs A = stage_args(c, ch);
+            A.R = std::max(1, kBatchTiles / A.G);
+            A.ntasks = (A.ngroups + A.R - 1) / A.R;
             A.src = st == 0 ? Aq : (st == 1 ? s1 : s2);
             A.fn = st == 0 ? nullptr : Aq;
             A.dst = st == 0 ? s1 : (st == 1 ? s2 : Aq);

@@ -74,10 +74,10 @@ struct StageArgs {
     int n1;              // nodes per direction (p + 1)
     int vt0;             // first global tile of the chunk
     int nvt;             // tiles in the chunk
-    int G;               // tiles per warp task and moment group
-    int T;               // tiles per CTA of k_stage3s (a multiple of G, set by its launch)
-    int group0;          // global index of the launch's first task group
-    int ngroups;         // task groups of the launch
+    int G;               // tiles per moment group
+    int R, ntasks;       // moment groups per task, tasks per element (plan_tasks)
+    int group0;          // global index of the launch's first moment group
+    int ngroups;         // moment groups of the launch
     // the velocity chunks of the launch (one, or all of them in a small problem's launch): chunk s holds local
     // tiles seg_vt[s] .. seg_vt[s+1] - 1 in groups seg_g[s] .. seg_g[s+1] - 1 (task_tiles)
     int nseg, seg_vt[10], seg_g[10];
@@ -108,6 +108,35 @@ struct StageArgs {
     const float *halo[2];
     int eface;           // elements on an x face (ne_y ne_z)
 };
+
+// Groups per task (R) and tasks of a launch over `units` elements (or element runs), `wave` of whose tasks are
+// resident at a time. A task writes its running moment sums out at the end of every group, so the partial sums
+// do not depend on R; longer tasks share the set-up and the first copies, which are not hidden behind the
+// task's own work (about `start` tiles' time), shorter ones leave less of the chip idle at the end (about
+// `tail` of a task). The rule takes the least of (tiles + start per task) / wave + tail of a task, or one
+// task's length where all are resident; start and tail are the kernel's, from sweeps of the task length (us per
+// launch): k_stage3s, 16^3 elements, 54 tiles: 1150 with 8 tiles per task, 1131 with 16, 1124 with 32, 1169
+// with 54; 315 elements, 42 tiles: 107 with 1, 95 with 2, 91 with 3 and 4, 96 with 6, 109 with 11; 90 elements,
+// 23 tiles: 32 with 1, 28 with 3, 37 with 6; k_stage3w, 2048 elements, 128 tiles: 740 with 8, 700 with 16, 692
+// with 32, 745 with 64.
+inline void plan_tasks(StageArgs &A, int64_t units, int64_t wave, double start, double tail)
+{
+    A.R = 1;
+    A.ntasks = A.ngroups;
+    if (A.nseg > 1)  // (several chunks in a small problem's launch: the groups as they are)
+        return;
+    double best = 0.0;
+    for (int r = 1; r <= A.ngroups; r++) {
+        const int tasks = (A.ngroups + r - 1) / r;
+        const double len = (double)(r * A.G < A.nvt ? r * A.G : A.nvt) + start;
+        const double cost = units * tasks <= wave ? len : units * (A.nvt + start * tasks) / (double)wave + tail * len;
+        if (r == 1 || cost < best) {
+            best = cost;
+            A.R = r;
+            A.ntasks = tasks;
+        }
+    }
+}
 
 struct NewtonArgs {
     const float *partial;  // [ngroups][5][n_x]

@@ -83,6 +83,7 @@ __device__ __forceinline__ void line_task(const StageArgs &A, const int task, co
     const int nr = ne * N1;  // real rows of the run
     int vl0, vl1;
     task_tiles(A, gl, vl0, vl1);
+    int ge = min(vl0 + A.G, vl1);  // end of the moment group
     int ec[3] = {eb, 0, 0};
     const int enL = upwind_neighbour(A.mesh, ec, 0, true);  // outside neighbours of the run
     ec[0] = eb + ne - 1;
@@ -298,19 +299,23 @@ __device__ __forceinline__ void line_task(const StageArgs &A, const int task, co
 #pragma unroll
             for (int c = 0; c < 5; c++)
                 msum[h][c] += sum2(pm[h][c]);
-    }
-    // partial moments of this task: combine the 4 velocity eighths of every row
-    const int grp = A.group0 + gl;
+        // the end of a moment group: combine the 4 velocity eighths of every row
+        if (vl + 1 == ge) {
+            const int grp = moment_group(A, task / nEB, vl);
 #pragma unroll
-    for (int h = 0; h < NHR; h++) {
-        const int row = np + 8 * h;
+            for (int h = 0; h < NHR; h++) {
+                const int row = np + 8 * h;
 #pragma unroll
-        for (int c = 0; c < 5; c++) {
-            float x = msum[h][c];
-            x += __shfl_xor_sync(0xffffffffu, x, 1);
-            x += __shfl_xor_sync(0xffffffffu, x, 2);
-            if (kg == 0 && row < nr)
-                A.partial[((int64_t)grp * 5 + c) * A.npts + (int64_t)eb * NP + row] = x;
+                for (int c = 0; c < 5; c++) {
+                    float x = msum[h][c];
+                    msum[h][c] = 0.f;
+                    x += __shfl_xor_sync(0xffffffffu, x, 1);
+                    x += __shfl_xor_sync(0xffffffffu, x, 2);
+                    if (kg == 0 && row < nr)
+                        A.partial[((int64_t)grp * 5 + c) * A.npts + (int64_t)eb * NP + row] = x;
+                }
+            }
+            ge = min(ge + A.G, vl1);
         }
     }
 }
@@ -320,7 +325,15 @@ template <int N1>
 __host__ __device__ int line_tasks(const StageArgs &A)
 {
     constexpr int K = line_run<N1>();
-    return ((A.mesh.nelem + K - 1) / K) * A.ngroups;
+    return ((A.mesh.nelem + K - 1) / K) * A.ntasks;
+}
+
+// Plan the tasks of a line launch (runs of elements, four warps per CTA).
+template <int N1>
+static void plan_line(StageArgs &A)
+{
+    constexpr int K = line_run<N1>();
+    plan_tasks(A, (A.mesh.nelem + K - 1) / K, 152 * BGK_LINE_MINCTAS * BGK_LINE_WARPS, 0.8, 1.0);
 }
 
 int stage1d_tasks(const StageArgs &A)
@@ -449,8 +462,10 @@ cudaError_t launch_stage3_p3(const StageArgs &A, int mode, int oct, cudaStream_t
 cudaError_t launch_stage2(const StageArgs &A, int p, int mode, int oct, cudaStream_t s);
 
 template <int N1>
-static cudaError_t launch_1d(const StageArgs &A, int mode, cudaStream_t s)
+static cudaError_t launch_1d(const StageArgs &A0, int mode, cudaStream_t s)
 {
+    StageArgs A = A0;
+    plan_line<N1>(A);
     const int ctas = (line_tasks<N1>(A) + BGK_LINE_WARPS - 1) / BGK_LINE_WARPS;
     const size_t smem = BGK_LINE_WARPS * sizeof(LineWarp<N1>);
     if (mode == 0)

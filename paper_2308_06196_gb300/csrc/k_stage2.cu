@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(kWarp *kWarpsPerCta, BGK_STAGE2_MINCTAS) k_sta
         return;  // the warps of a CTA never wait for one another
     QuadSmem<N1> &sm = smw[w];
     int vl0, vl1;
-    task_tiles(A, gl, vl0, vl1);
+    task_tiles(A, gl, vl0, vl1);  // one moment group per task (R = 1)
     const int ec[3] = {e % A.mesh.ne[0], e / A.mesh.ne[0], 0};
 
     if (MODE == 0) {
@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(kWarp *kWarpsPerCta, BGK_STAGE2_MINCTAS) k_sta
                 sm.msum[5 * h + c][lane] += sum2(pm[h][c]);
         __syncwarp();  // every lane is done with this tile's rows before they are refilled
     }
-    const int grp = A.group0 + gl;
+    const int grp = A.group0 + blockIdx.x / EB;
 #pragma unroll
     for (int h = 0; h < 2; h++) {
         const int q = np + 8 * h;

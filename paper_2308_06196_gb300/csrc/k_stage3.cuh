@@ -107,7 +107,9 @@ __device__ __forceinline__ void curv_line(float (&sv)[N1], const float (&fl)[N1]
 // reference-space flux (Ja^d . xi) f and per-lane upwinding at every face point from the shared face
 // normal, the element's neighbours, their shared faces and face-point orientations from its
 // connectivity row (curvilinear hexahedra on the structured element grid step in k_stage3c.cuh).
-template <int N1, int MODE, int OCT, int GEN, int CURV = 0>
+// SEG: the launch holds several chunks (the single-chunk form keeps the registers that the search would take: it
+// runs at its register limit, 322 against 325 us per octant launch of the random-order mesh below).
+template <int N1, int MODE, int OCT, int GEN, int CURV, int SEG>
 __global__ void __launch_bounds__(kWarp *N1, (N1 >= 4 ? (GEN || CURV ? BGK_STAGE3_MINCTAS_P3_GEN : BGK_STAGE3_MINCTAS_P3)
                                                : (N1 == 3 ? BGK_STAGE3_MINCTAS_P2 : 8))) k_stage3(const StageArgs A)
 {
@@ -124,8 +126,10 @@ __global__ void __launch_bounds__(kWarp *N1, (N1 >= 4 ? (GEN || CURV ? BGK_STAGE
     const int E = A.mesh.nelem;
     const int gl = blockIdx.x / E;
     const int e = blockIdx.x % E;
-    int vl0, vl1;
-    task_tiles(A, gl, vl0, vl1);
+    // one moment group per task (R = 1): see launch3
+    int vl0 = gl * A.G, vl1 = min(vl0 + A.G, A.nvt);
+    if constexpr (SEG)
+        task_tiles(A, gl, vl0, vl1);
     int ec[3];
     ec[0] = e % A.mesh.ne[0];
     ec[1] = (e / A.mesh.ne[0]) % A.mesh.ne[1];
@@ -617,7 +621,7 @@ __global__ void __launch_bounds__(kWarp *N1, (N1 >= 4 ? (GEN || CURV ? BGK_STAGE
         __syncwarp();
     }
     // partial moments of this task: combine the 4 velocity eighths of every node pair
-    const int grp = A.group0 + gl;
+    const int grp = A.group0 + blockIdx.x / E;
 #pragma unroll
     for (int h = 0; h < NHR; h++) {
         const int q = np + 8 * h;
@@ -633,19 +637,35 @@ __global__ void __launch_bounds__(kWarp *N1, (N1 >= 4 ? (GEN || CURV ? BGK_STAGE
 }
 
 
+// One moment group per task: with longer ones (plan_tasks) the elements in flight spread over more tiles and the
+// neighbour lines, read straight from global memory in whatever element order the mesh has, miss L2: 8^3
+// elements in random order at p = 3, 24^3 velocities, 324 -> 384 us per octant launch with two groups.
 template <int N1, int MODE, int OCT, int GEN, int CURV = 0>
 cudaError_t launch3(const StageArgs &A, cudaStream_t s)
 {
-    k_stage3<N1, MODE, OCT, GEN, CURV>
-        <<<A.mesh.nelem * A.ngroups, kWarp * N1, stage3_smem_bytes<N1, GEN, CURV>(), s>>>(A);
+    const int ctas = A.mesh.nelem * A.ngroups;
+    const size_t smem = stage3_smem_bytes<N1, GEN, CURV>();
+    if (A.nseg > 1)
+        k_stage3<N1, MODE, OCT, GEN, CURV, 1><<<ctas, kWarp * N1, smem, s>>>(A);
+    else
+        k_stage3<N1, MODE, OCT, GEN, CURV, 0><<<ctas, kWarp * N1, smem, s>>>(A);
     return cudaGetLastError();
+}
+
+// Shared-memory attribute of both forms of a k_stage3 kernel
+template <int N1, int MODE, int GEN, int CURV>
+cudaError_t prepare3_form()
+{
+    const int smem = (int)stage3_smem_bytes<N1, GEN, CURV>();
+    cudaError_t e = cudaFuncSetAttribute(k_stage3<N1, MODE, 8, GEN, CURV, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(k_stage3<N1, MODE, 8, GEN, CURV, 1>,
+                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
 template <int N1>
 cudaError_t prepare3()
 {
-    const int s0 = (int)sizeof(Stage3Smem<N1, 0>);
-    cudaError_t e = cudaFuncSetAttribute(k_stage3<N1, 1, 8, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, s0);
+    cudaError_t e = prepare3_form<N1, 1, 0, 0>();
     if constexpr (N1 <= 3) {
         if (e == cudaSuccess)
             e = prepare3w<N1>();
@@ -656,12 +676,9 @@ cudaError_t prepare3()
     if (e == cudaSuccess)
         e = prepare3c<N1>();
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_stage3<N1, 0, 8, 1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 stage3_smem_bytes<N1, 1, 2>());
+        e = prepare3_form<N1, 0, 1, 2>();
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_stage3<N1, 0, 8, 0, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 stage3_smem_bytes<N1, 0, 2>());
-
+        e = prepare3_form<N1, 0, 0, 2>();
     return e;
 }
 

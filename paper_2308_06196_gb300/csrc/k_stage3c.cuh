@@ -101,6 +101,7 @@ __global__ void __launch_bounds__(kWarp *N1, (N1 >= 4 ? BGK_STAGE3C_MINCTAS_P3 :
     const int e = blockIdx.x % E;
     int vl0, vl1;
     task_tiles(A, gl, vl0, vl1);
+    int ge = min(vl0 + A.G, vl1);  // end of the moment group
     int ec[3];
     ec[0] = e % A.mesh.ne[0];
     ec[1] = (e / A.mesh.ne[0]) % A.mesh.ne[1];
@@ -680,18 +681,22 @@ __global__ void __launch_bounds__(kWarp *N1, (N1 >= 4 ? BGK_STAGE3C_MINCTAS_P3 :
             octc = octn;
         }
         ka = ka == 2 ? 0 : ka + 1;
-    }
-    const int grp = A.group0 + gl;
+        if (vl + 1 == ge) {
+            const int grp = moment_group(A, blockIdx.x / E, vl);
 #pragma unroll
-    for (int h = 0; h < NHR; h++) {
-        const int q = np + 8 * h;
+            for (int h = 0; h < NHR; h++) {
+                const int q = np + 8 * h;
 #pragma unroll
-        for (int c = 0; c < 5; c++) {
-            float x = msum[h][c];
-            x += __shfl_xor_sync(0xffffffffu, x, 1);
-            x += __shfl_xor_sync(0xffffffffu, x, 2);
-            if (kg == 0 && q < NQ)
-                A.partial[((int64_t)grp * 5 + c) * A.npts + (int64_t)e * NP + q + NQ * w] = x;
+                for (int c = 0; c < 5; c++) {
+                    float x = msum[h][c];
+                    msum[h][c] = 0.f;
+                    x += __shfl_xor_sync(0xffffffffu, x, 1);
+                    x += __shfl_xor_sync(0xffffffffu, x, 2);
+                    if (kg == 0 && q < NQ)
+                        A.partial[((int64_t)grp * 5 + c) * A.npts + (int64_t)e * NP + q + NQ * w] = x;
+                }
+            }
+            ge = min(ge + A.G, vl1);
         }
     }
 }
@@ -747,14 +752,9 @@ __global__ void __launch_bounds__(kWarp *N1 / 2, 16) k_stage3cp(const StageArgs 
     const int lz = 2 * w + hf;                       // this lane's z-layer (and z-line slice iy)
     const int E = A.mesh.nelem;
     const int e = blockIdx.x % E;
-    int vl0, vl1, g0 = blockIdx.x / E;  // tiles, first moment group
-    if (A.T == A.G) {
-        task_tiles(A, g0, vl0, vl1);
-    } else {  // several groups of the launch's one chunk
-        vl0 = g0 * A.T;
-        vl1 = min(vl0 + A.T, A.nvt);
-        g0 = vl0 / A.G;
-    }
+    int vl0, vl1;
+    task_tiles(A, blockIdx.x / E, vl0, vl1);
+    int ge = min(vl0 + A.G, vl1);  // end of the moment group
     int ec[3];
     ec[0] = e % A.mesh.ne[0];
     ec[1] = (e / A.mesh.ne[0]) % A.mesh.ne[1];
@@ -1278,8 +1278,9 @@ __global__ void __launch_bounds__(kWarp *N1 / 2, 16) k_stage3cp(const StageArgs 
             fence_proxy_async();
             issue(ys, vl + 1, bF);
         }
-        if (!more || (vl + 1 - vl0) % A.G == 0) {  // the end of a moment group: combine the 4 velocity eighths of a row
-            const int grp = A.group0 + g0 + (vl - vl0) / A.G;
+        if (vl + 1 == ge) {  // the end of a moment group: combine the 4 velocity eighths of a row
+            const int grp = moment_group(A, blockIdx.x / E, vl);
+            ge = min(ge + A.G, vl1);
 #pragma unroll
             for (int r = 0; r < NR; r++)
 #pragma unroll
@@ -1334,10 +1335,11 @@ cudaError_t launch3c(const StageArgs &A0, cudaStream_t s)
                           offsetof(Sm, fnm) % 16 == 0 && offsetof(Sm, fpar) % 16 == 0 && offsetof(Sm, lim) % 16 == 0 &&
                           offsetof(Sm, bar) % 8 == 0,
                       "8- and 16-byte shared accesses");
-        const int ctas = stage3_tasks(A, 152 * 16);
-        k_stage3cp<N1, GEN><<<A.mesh.nelem * ctas, kWarp * N1 / 2, sizeof(Sm), s>>>(A);
+        plan_tasks(A, A.mesh.nelem, 152 * 16, 0.8, 1.0);
+        k_stage3cp<N1, GEN><<<A.mesh.nelem * A.ntasks, kWarp * N1 / 2, sizeof(Sm), s>>>(A);
     } else {
-        k_stage3c<N1, GEN><<<A.mesh.nelem * A.ngroups, kWarp * N1, sizeof(Stage3cSmem<N1, GEN>), s>>>(A);
+        plan_tasks(A, A.mesh.nelem, 152 * (N1 >= 4 ? BGK_STAGE3C_MINCTAS_P3 : 6), 0.8, 0.5);
+        k_stage3c<N1, GEN><<<A.mesh.nelem * A.ntasks, kWarp * N1, sizeof(Stage3cSmem<N1, GEN>), s>>>(A);
     }
     return cudaGetLastError();
 }

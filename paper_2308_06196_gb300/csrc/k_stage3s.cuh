@@ -38,8 +38,7 @@ namespace bgk {
 // elements 63.3 -> 58.0 ms.
 // Warp 0 also brings the tile's velocity table into a double-buffered block with a barrier of its own, which
 // every warp waits on. No global load is left in the tile loop of the periodic form.
-// A CTA runs T tiles, a multiple of the G tiles of a moment group: it writes its running moment sums out
-// every G tiles, so the partial sums do not depend on T.
+// A CTA runs R moment groups of G tiles and writes its running moment sums out after each (plan_tasks).
 // ------------------------------------------------------------------------------------------------
 // velocity table rows per tile: the grid indices m_x, m_y, m_z, the index-basis weight W (0 on padded
 // slots) and the energy weight W sum_d r_d m_d^2; the moment weights W m_d are formed from them (exact)
@@ -86,14 +85,9 @@ __global__ void __launch_bounds__(kWarp *N1 / 2, kStage3sCtas<GEN>)
     const int lz = 2 * w + hf;                       // this lane's z-layer (and z-line slice iy)
     const int E = A.mesh.nelem;
     const int e = blockIdx.x % E;
-    int vl0, vl1, g0 = blockIdx.x / E;  // tiles, first moment group
-    if (A.T == A.G) {
-        task_tiles(A, g0, vl0, vl1);
-    } else {  // several groups of the launch's one chunk
-        vl0 = g0 * A.T;
-        vl1 = min(vl0 + A.T, A.nvt);
-        g0 = vl0 / A.G;
-    }
+    int vl0, vl1;
+    task_tiles(A, blockIdx.x / E, vl0, vl1);
+    int ge = min(vl0 + A.G, vl1);  // end of the moment group
     int ec[3];
     ec[0] = e % A.mesh.ne[0];
     ec[1] = (e / A.mesh.ne[0]) % A.mesh.ne[1];
@@ -530,8 +524,9 @@ __global__ void __launch_bounds__(kWarp *N1 / 2, kStage3sCtas<GEN>)
             fence_proxy_async();
             issue(ys, vl + 1, bF);
         }
-        if (!more || (vl + 1 - vl0) % A.G == 0) {  // the end of a moment group: combine the 4 velocity eighths of a row
-            const int grp = A.group0 + g0 + (vl - vl0) / A.G;
+        if (vl + 1 == ge) {  // the end of a moment group: combine the 4 velocity eighths of a row
+            const int grp = moment_group(A, blockIdx.x / E, vl);
+            ge = min(ge + A.G, vl1);
 #pragma unroll
             for (int r = 0; r < NR; r++)
 #pragma unroll
@@ -555,18 +550,6 @@ __global__ void __launch_bounds__(kWarp *N1 / 2, kStage3sCtas<GEN>)
     }
 }
 
-// Tiles per CTA (A.T): as many whole moment groups as leave eight waves of `wave` CTAs (a CTA's first copies are
-// not hidden behind its own work: 16^3 elements, 54 tiles per octant, ran 3 % faster with 32 tiles per CTA
-// than with 8). Returns the CTAs per element.
-inline int stage3_tasks(StageArgs &A, int wave)
-{
-    const int64_t E = A.mesh.nelem;
-    A.T = A.G;
-    while (A.nseg == 1 && A.T < A.nvt && E * ((A.nvt + 2 * A.T - 1) / (2 * A.T)) >= 8 * wave)
-        A.T *= 2;
-    return A.T == A.G ? A.ngroups : (A.nvt + A.T - 1) / A.T;
-}
-
 template <int N1, int OCT, int GEN>
 cudaError_t launch3s(const StageArgs &A0, cudaStream_t s)
 {
@@ -575,8 +558,8 @@ cudaError_t launch3s(const StageArgs &A0, cudaStream_t s)
                       offsetof(Sm, lim) % 16 == 0 && offsetof(Sm, bar) % 8 == 0,
                   "8- and 16-byte shared accesses");
     StageArgs A = A0;
-    const int ctas = stage3_tasks(A, 152 * kStage3sCtas<GEN>);
-    k_stage3s<N1, OCT, GEN><<<A.mesh.nelem * ctas, kWarp * N1 / 2, sizeof(Sm), s>>>(A);
+    plan_tasks(A, A.mesh.nelem, 152 * kStage3sCtas<GEN>, 0.8, 0.7);
+    k_stage3s<N1, OCT, GEN><<<A.mesh.nelem * A.ntasks, kWarp * N1 / 2, sizeof(Sm), s>>>(A);
     return cudaGetLastError();
 }
 

@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(kWarp *BGK_STAGE3W_WARPS, (N1 == 3 ? BGK_STAGE
         return;
     int vl0, vl1;
     task_tiles(A, gl, vl0, vl1);
+    int ge = min(vl0 + A.G, vl1);  // end of the moment group
     int ec[3];
     ec[0] = e % A.mesh.ne[0];
     ec[1] = (e / A.mesh.ne[0]) % A.mesh.ne[1];
@@ -471,28 +472,34 @@ __global__ void __launch_bounds__(kWarp *BGK_STAGE3W_WARPS, (N1 == 3 ? BGK_STAGE
         for (int d = 0; d < 3; d++)
             en[d] = enn[d];
         ka = ka == 2 ? 0 : ka + 1;
-    }
-    // partial moments of this task: combine the 4 velocity eighths of every row
-    const int grp = A.group0 + gl;
+        // the end of a moment group: combine the 4 velocity eighths of every row
+        if (vl + 1 == ge) {
+            const int grp = moment_group(A, blockIdx.x / nblk, vl);
 #pragma unroll
-    for (int h = 0; h < NHR; h++) {
-        const int q = np + 8 * h;
+            for (int h = 0; h < NHR; h++) {
+                const int q = np + 8 * h;
 #pragma unroll
-        for (int c = 0; c < 5; c++) {
-            float x = msum[h][c];
-            x += __shfl_xor_sync(0xffffffffu, x, 1);
-            x += __shfl_xor_sync(0xffffffffu, x, 2);
-            if (kg == 0 && q < NP)
-                A.partial[((int64_t)grp * 5 + c) * A.npts + (int64_t)e * NP + q] = x;
+                for (int c = 0; c < 5; c++) {
+                    float x = msum[h][c];
+                    msum[h][c] = 0.f;
+                    x += __shfl_xor_sync(0xffffffffu, x, 1);
+                    x += __shfl_xor_sync(0xffffffffu, x, 2);
+                    if (kg == 0 && q < NP)
+                        A.partial[((int64_t)grp * 5 + c) * A.npts + (int64_t)e * NP + q] = x;
+                }
+            }
+            ge = min(ge + A.G, vl1);
         }
     }
 }
 
 template <int N1, int OCT, int GEN>
-cudaError_t launch3w(const StageArgs &A, cudaStream_t s)
+cudaError_t launch3w(const StageArgs &A0, cudaStream_t s)
 {
+    StageArgs A = A0;
+    plan_tasks(A, A.mesh.nelem, 152 * (N1 == 3 ? BGK_STAGE3W_MINCTAS_P2 : 16), 2.0, 0.5);
     const int nblk = (A.mesh.nelem + BGK_STAGE3W_WARPS - 1) / BGK_STAGE3W_WARPS;
-    k_stage3w<N1, OCT, GEN><<<nblk * A.ngroups, kWarp * BGK_STAGE3W_WARPS,
+    k_stage3w<N1, OCT, GEN><<<nblk * A.ntasks, kWarp * BGK_STAGE3W_WARPS,
                               BGK_STAGE3W_WARPS * sizeof(Stage3wWarp<N1, GEN>), s>>>(A);
     return cudaGetLastError();
 }

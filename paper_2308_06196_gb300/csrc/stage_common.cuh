@@ -4,20 +4,27 @@
 
 namespace bgk {
 
-// Tiles [vl0, vl1) of task group gl of a launch: groups of G tiles that do not cross a chunk's end, so the
-// partial moment sums are the same whether the chunks are launched one by one or together.
-__device__ __forceinline__ void task_tiles(const StageArgs &A, int gl, int &vl0, int &vl1)
+// Tiles [vl0, vl1) of task t of a launch: R groups of G tiles that do not cross a chunk's end (one group in a
+// launch over several chunks), so the partial moment sums are the same however the chunks are launched and
+// the groups are shared out.
+__device__ __forceinline__ void task_tiles(const StageArgs &A, int t, int &vl0, int &vl1)
 {
-    if (A.nseg == 1) {  // (the usual launch: no search, which a short task would feel)
-        vl0 = gl * A.G;
-        vl1 = min(vl0 + A.G, A.nvt);
+    if (__builtin_expect(A.nseg == 1, 1)) {  // no search, which a short task would feel
+        vl0 = t * A.R * A.G;
+        vl1 = min(vl0 + A.R * A.G, A.nvt);
         return;
     }
     int s = 0;
-    while (s + 1 < A.nseg && gl >= A.seg_g[s + 1])
+    while (s + 1 < A.nseg && t >= A.seg_g[s + 1])
         s++;
-    vl0 = A.seg_vt[s] + (gl - A.seg_g[s]) * A.G;
+    vl0 = A.seg_vt[s] + (t - A.seg_g[s]) * A.G;
     vl1 = min(vl0 + A.G, A.seg_vt[s + 1]);
+}
+
+// The moment group of tile vl of task t
+__device__ __forceinline__ int moment_group(const StageArgs &A, int t, int vl)
+{
+    return A.group0 + (A.nseg == 1 ? vl / A.G : t);
 }
 
 // fused multiply-add on two packed FP32 lanes (sm_100+): d = a * b + c, element-wise
