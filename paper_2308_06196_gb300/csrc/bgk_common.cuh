@@ -111,25 +111,28 @@ struct StageArgs {
 
 // Groups per task (R) and tasks of a launch over `units` elements (or element runs), `wave` of whose tasks are
 // resident at a time. A task writes its running moment sums out at the end of every group, so the partial sums
-// do not depend on R; longer tasks share the set-up and the first copies, which are not hidden behind the
-// task's own work (about `start` tiles' time), shorter ones leave less of the chip idle at the end (about
-// `tail` of a task). The rule takes the least of (tiles + start per task) / wave + tail of a task, or one
-// task's length where all are resident; start and tail are the kernel's, from sweeps of the task length (us per
-// launch): k_stage3s, 16^3 elements, 54 tiles: 1150 with 8 tiles per task, 1131 with 16, 1124 with 32, 1169
-// with 54; 315 elements, 42 tiles: 107 with 1, 95 with 2, 91 with 3 and 4, 96 with 6, 109 with 11; 90 elements,
-// 23 tiles: 32 with 1, 28 with 3, 37 with 6; k_stage3w, 2048 elements, 128 tiles: 740 with 8, 700 with 16, 692
-// with 32, 745 with 64.
-inline void plan_tasks(StageArgs &A, int64_t units, int64_t wave, double start, double tail)
+// do not depend on R. Longer tasks share the set-up and the first copies, which are not hidden behind the
+// task's own work (about `start` tiles' time); shorter ones leave less of the chip idle in the last round,
+// which takes idle + (1 - idle) x of a full one's time when it is filled to x. The rule takes the least of
+//   (tiles + start per task) units / wave + what the last round wastes of a task's length;
+// start and idle are the kernel's, from sweeps of the task length (tiles per task: us per launch). k_stage3s:
+// 16^3 elements, 54 tiles, 8: 1150, 16: 1131, 32: 1124, 54: 1169; 315 elements, 42 tiles, 1: 107, 2: 95, 3: 91,
+// 4: 91, 6: 96, 11: 109; 90 elements, 23 tiles, 1: 32, 3: 28, 6: 37. k_stage3w: 2048 elements, 128 tiles, 8: 740,
+// 16: 700, 32: 692, 64: 745; 360 elements, 69 to 86 tiles, 2: 100, 4: 92, 8: 89, 12: 103, 16: 87, 22: 105.
+inline void plan_tasks(StageArgs &A, int64_t units, int64_t wave, double start, double idle)
 {
     A.R = 1;
     A.ntasks = A.ngroups;
     if (A.nseg > 1)  // (several chunks in a small problem's launch: the groups as they are)
         return;
+    auto last = [&](double x) { return x > 0.0 ? idle + (1.0 - idle) * x : 0.0; };
     double best = 0.0;
     for (int r = 1; r <= A.ngroups; r++) {
         const int tasks = (A.ngroups + r - 1) / r;
         const double len = (double)(r * A.G < A.nvt ? r * A.G : A.nvt) + start;
-        const double cost = units * tasks <= wave ? len : units * (A.nvt + start * tasks) / (double)wave + tail * len;
+        const double rounds = (double)(units * tasks) / (double)wave, part = rounds - (double)(int64_t)rounds;
+        const double cost = rounds <= 1.0 ? 1.1 * last(rounds) * len  // (nothing left to balance the SMs with)
+                                          : units * (A.nvt + start * tasks) / (double)wave + (last(part) - part) * len;
         if (r == 1 || cost < best) {
             best = cost;
             A.R = r;

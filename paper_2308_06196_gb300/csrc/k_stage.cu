@@ -333,7 +333,7 @@ template <int N1>
 static void plan_line(StageArgs &A)
 {
     constexpr int K = line_run<N1>();
-    plan_tasks(A, (A.mesh.nelem + K - 1) / K, 152 * BGK_LINE_MINCTAS * BGK_LINE_WARPS, 0.8, 1.0);
+    plan_tasks(A, (A.mesh.nelem + K - 1) / K, 152 * BGK_LINE_MINCTAS * BGK_LINE_WARPS, 0.8, 0.6);
 }
 
 int stage1d_tasks(const StageArgs &A)

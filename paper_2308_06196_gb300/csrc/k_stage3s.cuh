@@ -558,7 +558,7 @@ cudaError_t launch3s(const StageArgs &A0, cudaStream_t s)
                       offsetof(Sm, lim) % 16 == 0 && offsetof(Sm, bar) % 8 == 0,
                   "8- and 16-byte shared accesses");
     StageArgs A = A0;
-    plan_tasks(A, A.mesh.nelem, 152 * kStage3sCtas<GEN>, 0.8, 0.7);
+    plan_tasks(A, A.mesh.nelem, 152 * kStage3sCtas<GEN>, 0.8, 0.75);
     k_stage3s<N1, OCT, GEN><<<A.mesh.nelem * A.ntasks, kWarp * N1 / 2, sizeof(Sm), s>>>(A);
     return cudaGetLastError();
 }

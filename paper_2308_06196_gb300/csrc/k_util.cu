@@ -126,8 +126,8 @@ __global__ void __launch_bounds__(256, 4)
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     // the tile's table columns (1 + k_x, 1 + n_x + k_y, 1 + n_x + n_y + k_z) from the centred index table
-    // (k_d = (m_d + n_d - 1) / 2, exact), column 0 on padded slots; the next tile's are loaded while this one
-    // is written
+    // (k_d = (m_d + n_d - 1) / 2, exact), column 0 on padded slots; the warp's next tile's are loaded while
+    // this one is written
     auto slot_cols = [&](int vt, int &cx, int &cy, int &cz) {
         const int slot = vt * kWarp + lane;
         cx = 1 + __float2int_rn(0.5f * (__ldg(mi + slot) + (float)(nx - 1)));
@@ -136,21 +136,22 @@ __global__ void __launch_bounds__(256, 4)
         if (__ldg(gmask + slot) == 0.f)
             cx = 0;
     };
-    const int vt0 = blockIdx.y * tiles, vt1 = min(vt0 + tiles, nvt);
-    if (vt0 >= vt1)
+    // a warp per tile, all of the CTA's points: the tile's columns are loaded once and serve PB rows
+    const int vt1 = min((int)(blockIdx.y + 1) * tiles, nvt);
+    int vt = blockIdx.y * tiles + w;
+    if (vt >= vt1)
         return;
     int cx, cy, cz;
-    slot_cols(vt0, cx, cy, cz);
-    for (int vt = vt0; vt < vt1; vt++) {
+    slot_cols(vt, cx, cy, cz);
+    for (; vt < vt1; vt += nw) {
         int nx_ = 0, ny_ = 0, nz_ = 0;
-        if (vt + 1 < vt1)
-            slot_cols(vt + 1, nx_, ny_, nz_);
+        if (vt + nw < vt1)
+            slot_cols(vt + nw, nx_, ny_, nz_);
         float *dst = f + ((int64_t)vt * npts + p0) * kWarp + lane;
-#pragma unroll 4
-        for (int i = w; i < np; i += nw) {
-            const float *t = tab + i * ntab;
-            __stcs(dst + i * kWarp, t[cx] * t[cy] * t[cz]);
-        }
+        const float *tx = tab + cx, *ty = tab + cy, *tz = tab + cz;
+#pragma unroll 8
+        for (int i = 0; i < np; i++)
+            __stcs(dst + i * kWarp, tx[i * ntab] * ty[i * ntab] * tz[i * ntab]);
         cx = nx_;
         cy = ny_;
         cz = nz_;
