@@ -20,13 +20,26 @@ namespace bgk {
 // Bound: the tables by the FP64 pipe (a warp instruction per 16 clocks, whatever its active lanes), the
 // values by the writing of f. One CTA per element left most lanes of the table and moment work idle at
 // four points per element, and a small mesh's tiles to a few CTAs. 65,536 line elements at p = 3, 32^2
-// velocities (1.1 GB of f): 3.24 ms before, 1.00 now; 128^2 quadrilaterals 1.37 -> 1.00; 16^3
-// hexahedra, 24^3 velocities (14.5 GB) 3.34 -> 3.25.
+// velocities (1.1 GB of f): 3.24 ms before, 0.61 now; 128^2 quadrilaterals 1.37 -> 0.61; 16^3
+// hexahedra, 24^3 velocities (14.5 GB) 3.34 -> 2.02.
+// (n = rint(y) by the rounding constant 1.5 2^52, whose low word then holds n: two FP64 operations for three
+// and a conversion. Below 2^-2000 the result is 0 anyway and n would not fit.)
 __device__ __forceinline__ float exp_split(double x)
 {
-    const double y = x * 1.4426950408889634;  // log2(e)
-    const double n = rint(y);
-    return ldexpf(exp2f((float)(y - n)), (int)n);
+    const double y = x * 1.4426950408889634;  // log2(e); y <= 0
+    if ((unsigned)__double2hiint(y) > 0xc09f4000u)  // y < -2000, or NaN
+        return y < 0.0 ? 0.f : (float)y;
+    const double t = __dadd_rn(y, 6755399441055744.0);
+    const double n = __dsub_rn(t, 6755399441055744.0);
+    return ldexpf(exp2f((float)(y - n)), __double2loint(t));
+}
+// the exact double of a non-negative FP32 value without the FP64 pipe's conversion
+__device__ __forceinline__ double widen(float v)
+{
+    const unsigned u = __float_as_uint(v);
+    if (u - 0x00800000u >= 0x7f000000u)  // zero, subnormal, infinite or NaN
+        return (double)v;
+    return __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29));
 }
 
 __global__ void __launch_bounds__(256, 4)
@@ -39,7 +52,9 @@ __global__ void __launch_bounds__(256, 4)
     const int ntab = nx + ny + nz + 1;       // per point: 0 (padded slots), then the factors by axis
     extern __shared__ double ith[];          // [PB] -1 / (2 theta) of the CTA's points,
     double *S = ith + PB;                    // [PB][3][3] 1-D sums,
-    float *cn = reinterpret_cast<float *>(S + 9 * PB);  // [PB] normalisations,
+    double *xg = S + 9 * PB;                 // [ntab - 1] velocities of the nodes, axis by axis,
+    double *x2 = xg + (ntab - 1);            // [ntab - 1] and their squares,
+    float *cn = reinterpret_cast<float *>(x2 + (ntab - 1));  // [PB] normalisations,
     float *tab = cn + PB;                    // [PB][ntab]
     const int p0 = blockIdx.x * PB, np = min(PB, npts - p0);
     const bool first = blockIdx.y == 0;      // writes the points' moments and warm starts
@@ -63,25 +78,21 @@ __global__ void __launch_bounds__(256, 4)
             wp[4] = th;
         }
     }
+    for (int t = threadIdx.x; t < ntab - 1; t += blockDim.x) {
+        const int d = t < nx ? 0 : (t < nx + ny ? 1 : 2), k = t - (d > 0 ? nx : 0) - (d > 1 ? ny : 0);
+        xg[t] = fma((double)k, d == 0 ? dvx : (d == 1 ? dvy : dvz), d == 0 ? v0x : (d == 1 ? v0y : v0z));
+        x2[t] = xg[t] * xg[t];
+    }
     __syncthreads();
     for (int q = threadIdx.x; q < np * (ntab - 1); q += blockDim.x) {
-        const int i = q / (ntab - 1), t = 1 + q % (ntab - 1);
-        const double *s = prim + (int64_t)(p0 + i) * 5;
+        const int i = q / (ntab - 1), t = q % (ntab - 1);
         const double a = ith[i];
-        float v;
-        if (t <= nx) {
-            const double c = v0x + (t - 1) * dvx - s[1];
-            v = exp_split(a * c * c);
-        } else if (t <= nx + ny) {
-            const double c = v0y + (t - 1 - nx) * dvy - s[2];
-            v = exp_split(a * c * c);
-        } else if (nz == 1) {
-            v = 1.f;
-        } else {
-            const double c = v0z + (t - 1 - nx - ny) * dvz - s[3];
+        float v = 1.f;
+        if (t < nx + ny || nz > 1) {
+            const double c = xg[t] - prim[(int64_t)(p0 + i) * 5 + (t < nx ? 1 : (t < nx + ny ? 2 : 3))];
             v = exp_split(a * c * c);
         }
-        tab[i * ntab + t] = a == 0.0 ? 0.f : v;
+        tab[i * ntab + 1 + t] = a == 0.0 ? 0.f : v;
     }
     __syncthreads();
     if (Q && first) {
@@ -89,24 +100,24 @@ __global__ void __launch_bounds__(256, 4)
         for (int q = threadIdx.x; q < 3 * np; q += blockDim.x) {
             const int d = q / np, i = q % np;
             const int n = d == 0 ? nx : (d == 1 ? ny : nz);
-            const double v0 = d == 0 ? v0x : (d == 1 ? v0y : v0z), dv = d == 0 ? dvx : (d == 1 ? dvy : dvz);
-            const float *t = tab + i * ntab + 1 + (d > 0 ? nx : 0) + (d > 1 ? ny : 0);
+            const double dv = d == 0 ? dvx : (d == 1 ? dvy : dvz), hv = 0.5 * dv;
+            const int o = (d > 0 ? nx : 0) + (d > 1 ? ny : 0);
+            const float *t = tab + i * ntab + 1 + o;
             double s0 = 0.0, s1 = 0.0, s2 = 0.0;
             if (n == 1) {  // the absent u_z: one node at 0 of unit weight
                 s0 = (double)t[0];
             } else {
                 for (int k = 0; k < n; k++) {
-                    const double x = v0 + k * dv;
-                    const double a = (k == 0 || k == n - 1 ? 0.5 * dv : dv) * (double)t[k];
+                    const double a = (k == 0 || k == n - 1 ? hv : dv) * widen(t[k]);
                     s0 += a;
-                    s1 = fma(x, a, s1);
-                    s2 = fma(x * x, a, s2);
+                    s1 = fma(xg[o + k], a, s1);
+                    s2 = fma(x2[o + k], a, s2);
                 }
             }
-            double *o = S + (i * 3 + d) * 3;
-            o[0] = s0;
-            o[1] = s1;
-            o[2] = s2;
+            double *so = S + (i * 3 + d) * 3;
+            so[0] = s0;
+            so[1] = s1;
+            so[2] = s2;
         }
         __syncthreads();
         for (int i = threadIdx.x; i < np; i += blockDim.x) {
@@ -198,9 +209,10 @@ cudaError_t launch_init_maxwellian(float *f, const double *prim, const float *mi
     // points per CTA: 64, so that two warps of them fill the lanes of the FP64 work, but 32 where that leaves
     // fewer than two CTAs per SM, and no more than 96 KB of tables (two CTAs per SM) where the grid allows
     const int per = 10 * (int)sizeof(double) + (ntab + 1) * (int)sizeof(float);
+    const int grid = 2 * (ntab - 1) * (int)sizeof(double);
     int PB = npts >= 64 * 304 ? 64 : 32;
-    PB = std::max(1, std::min(PB, 98304 / per));
-    const int smem = PB * per;
+    PB = std::max(1, std::min(PB, (98304 - grid) / per));
+    const int smem = PB * per + grid;
     // runs of at least 32 tiles (their writing outweighs the tables that every run forms anew), as many as
     // two CTAs per SM take
     const int nb = (npts + PB - 1) / PB;
