@@ -1,4 +1,5 @@
-// k_stage2.cu -- the fused SSP-RK3 stage kernel for quadrilaterals (dim = 2, FP32-split form): the
+// k_stage2.cu -- the fused SSP-RK3 stage kernel for quadrilaterals (dim = 2, FP32-split form) of odd line
+// length (p = 2; the even ones step in k_stage2p) and the moments-only pass of all: the
 // planar problems of the method (Sec. 2 with d = 2, velocity dimension m = 2 or 3).
 //
 // One CTA per (block of 4 elements, run of G tiles); warp w owns element 4 b + w and works alone (no
@@ -7,7 +8,7 @@
 // in shared memory with cp.async one tile ahead, f^n is refilled after use; the upwind neighbours'
 // lines come from L2. The Maxwellian, the Shu-Osher combination, the positivity limiter (in registers:
 // the element is the warp's) and the moment sums of the stored output follow as in the hexahedral kernel.
-#include "stage_common.cuh"
+#include "k_stage2p.cuh"
 
 namespace bgk {
 
@@ -30,6 +31,7 @@ struct alignas(16) QuadSmem {
 template <int N1, int MODE, int OCT>
 __global__ void __launch_bounds__(kWarp *kWarpsPerCta, BGK_STAGE2_MINCTAS) k_stage2(const StageArgs A)
 {
+    static_assert(MODE == 1 || N1 % 2 == 1, "even line lengths step in k_stage2p");
     constexpr int NQ = N1 * N1;
     constexpr int NCH = NQ * kWarp / 4;  // 16-byte chunks of one element tile
     __shared__ QuadSmem<N1> smw[kWarpsPerCta];
@@ -168,95 +170,39 @@ __global__ void __launch_bounds__(kWarp *kWarpsPerCta, BGK_STAGE2_MINCTAS) k_sta
                 acc[q] = fmaf(A.an, acc[q], kbq * f[q]);
             }
             const float cx = -A.mesh.inv_h2[0] * x0 * bdt, cy = -A.mesh.inv_h2[1] * x1 * bdt;
-            if constexpr (N1 % 2 == 0) {
-                // two adjacent lines of a direction at a time on packed FP32 pairs, the upwind value in
-                // jump form inside the trace (as the hexahedral kernels), selected against the ghost jump
-                constexpr int RL = 0, RR = N1 - 1;
 #pragma unroll
-                for (int iy = 0; iy < N1; iy += 2) {
-                    unsigned long long fl[N1], v[N1], sv[N1];
+            for (int iy = 0; iy < N1; iy++) {
+                float fl[N1], sv[N1];
 #pragma unroll
-                    for (int j = 0; j < N1; j++) {
-                        fl[j] = pack2(f[j + N1 * iy], f[j + N1 * iy + N1]);
-                        v[j] = pack2(vx[iy][j], vx[iy + 1][j]);
-                    }
-                    if (l0) {
-                        const unsigned long long tj = trace_jump2<N1, true>(v, fl[RL], A.ops);
-                        const unsigned long long gj = fsub2(dup2(gx), fl[RL]);
-                        line_sums_jump2<N1, true>(sv, fl, enx >= 0 ? tj : gj, A.ops);
-                    } else {
-                        const unsigned long long tj = trace_jump2<N1, false>(v, fl[RR], A.ops);
-                        const unsigned long long gj = fsub2(dup2(gx), fl[RR]);
-                        line_sums_jump2<N1, false>(sv, fl, enx >= 0 ? tj : gj, A.ops);
-                    }
-#pragma unroll
-                    for (int j = 0; j < N1; j++) {
-                        float lo, hi;
-                        unpack2(sv[j], lo, hi);
-                        acc[j + N1 * iy] = fmaf(cx, lo, acc[j + N1 * iy]);
-                        acc[j + N1 * iy + N1] = fmaf(cx, hi, acc[j + N1 * iy + N1]);
-                    }
+                for (int j = 0; j < N1; j++)
+                    fl[j] = f[j + N1 * iy];
+                if (l0) {
+                    const float t = trace_line<N1, true>(vx[iy], A.ops);
+                    line_sums<N1, true>(sv, fl, enx >= 0 ? t : gx, A.ops);
+                } else {
+                    const float t = trace_line<N1, false>(vx[iy], A.ops);
+                    line_sums<N1, false>(sv, fl, enx >= 0 ? t : gx, A.ops);
                 }
 #pragma unroll
-                for (int ix = 0; ix < N1; ix += 2) {
-                    unsigned long long fl[N1], v[N1], sv[N1];
+                for (int j = 0; j < N1; j++)
+                    acc[j + N1 * iy] = fmaf(cx, sv[j], acc[j + N1 * iy]);
+            }
 #pragma unroll
-                    for (int j = 0; j < N1; j++) {
-                        fl[j] = pack2(f[ix + N1 * j], f[ix + 1 + N1 * j]);
-                        v[j] = pack2(vy[ix][j], vy[ix + 1][j]);
-                    }
-                    if (l1) {
-                        const unsigned long long tj = trace_jump2<N1, true>(v, fl[RL], A.ops);
-                        const unsigned long long gj = fsub2(dup2(gy), fl[RL]);
-                        line_sums_jump2<N1, true>(sv, fl, eny >= 0 ? tj : gj, A.ops);
-                    } else {
-                        const unsigned long long tj = trace_jump2<N1, false>(v, fl[RR], A.ops);
-                        const unsigned long long gj = fsub2(dup2(gy), fl[RR]);
-                        line_sums_jump2<N1, false>(sv, fl, eny >= 0 ? tj : gj, A.ops);
-                    }
+            for (int ix = 0; ix < N1; ix++) {
+                float fl[N1], sv[N1];
 #pragma unroll
-                    for (int j = 0; j < N1; j++) {
-                        float lo, hi;
-                        unpack2(sv[j], lo, hi);
-                        acc[ix + N1 * j] = fmaf(cy, lo, acc[ix + N1 * j]);
-                        acc[ix + 1 + N1 * j] = fmaf(cy, hi, acc[ix + 1 + N1 * j]);
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int iy = 0; iy < N1; iy++) {
-                    float fl[N1], sv[N1];
-#pragma unroll
-                    for (int j = 0; j < N1; j++)
-                        fl[j] = f[j + N1 * iy];
-                    if (l0) {
-                        const float t = trace_line<N1, true>(vx[iy], A.ops);
-                        line_sums<N1, true>(sv, fl, enx >= 0 ? t : gx, A.ops);
-                    } else {
-                        const float t = trace_line<N1, false>(vx[iy], A.ops);
-                        line_sums<N1, false>(sv, fl, enx >= 0 ? t : gx, A.ops);
-                    }
-#pragma unroll
-                    for (int j = 0; j < N1; j++)
-                        acc[j + N1 * iy] = fmaf(cx, sv[j], acc[j + N1 * iy]);
+                for (int j = 0; j < N1; j++)
+                    fl[j] = f[ix + N1 * j];
+                if (l1) {
+                    const float t = trace_line<N1, true>(vy[ix], A.ops);
+                    line_sums<N1, true>(sv, fl, eny >= 0 ? t : gy, A.ops);
+                } else {
+                    const float t = trace_line<N1, false>(vy[ix], A.ops);
+                    line_sums<N1, false>(sv, fl, eny >= 0 ? t : gy, A.ops);
                 }
 #pragma unroll
-                for (int ix = 0; ix < N1; ix++) {
-                    float fl[N1], sv[N1];
-#pragma unroll
-                    for (int j = 0; j < N1; j++)
-                        fl[j] = f[ix + N1 * j];
-                    if (l1) {
-                        const float t = trace_line<N1, true>(vy[ix], A.ops);
-                        line_sums<N1, true>(sv, fl, eny >= 0 ? t : gy, A.ops);
-                    } else {
-                        const float t = trace_line<N1, false>(vy[ix], A.ops);
-                        line_sums<N1, false>(sv, fl, eny >= 0 ? t : gy, A.ops);
-                    }
-#pragma unroll
-                    for (int j = 0; j < N1; j++)
-                        acc[ix + N1 * j] = fmaf(cy, sv[j], acc[ix + N1 * j]);
-                }
+                for (int j = 0; j < N1; j++)
+                    acc[ix + N1 * j] = fmaf(cy, sv[j], acc[ix + N1 * j]);
             }
             // BGK source towards the conservative Maxwellian and the Shu-Osher combination, two nodes at
             // a time (exponent a + b.m + q |m|^2, or per-axis q on grids of several spacings)
@@ -378,16 +324,36 @@ cudaError_t launch2(const StageArgs &A, cudaStream_t s)
     return cudaGetLastError();
 }
 
+template <int N1, int GEN>
+cudaError_t launch2p_oct(const StageArgs &A, int oct, cudaStream_t s)
+{
+    if (oct >= 8)
+        return launch2p<N1, 8, GEN>(A, s);
+    switch (oct & 3) {  // the z sign takes no part in a planar advection
+    case 0: return launch2p<N1, 0, GEN>(A, s);
+    case 1: return launch2p<N1, 1, GEN>(A, s);
+    case 2: return launch2p<N1, 2, GEN>(A, s);
+    default: return launch2p<N1, 3, GEN>(A, s);
+    }
+}
+
 template <int N1>
 cudaError_t launch2_any(const StageArgs &A, int mode, int oct, cudaStream_t s)
 {
     if (mode == 1)
         return launch2<N1, 1, 8>(A, s);
-    switch (oct & 3) {  // the z sign takes no part in a planar advection
-    case 0: return oct < 8 ? launch2<N1, 0, 0>(A, s) : launch2<N1, 0, 8>(A, s);
-    case 1: return oct < 8 ? launch2<N1, 0, 1>(A, s) : launch2<N1, 0, 8>(A, s);
-    case 2: return oct < 8 ? launch2<N1, 0, 2>(A, s) : launch2<N1, 0, 8>(A, s);
-    default: return oct < 8 ? launch2<N1, 0, 3>(A, s) : launch2<N1, 0, 8>(A, s);
+    if constexpr (N1 % 2 == 0) {  // even line length: packed pairs of velocities
+        bool general = !A.viso || A.limiter || A.vtau;
+        for (int f = 0; f < 4; f++)
+            general = general || A.mesh.bc[f] != 0;
+        return general ? launch2p_oct<N1, 1>(A, oct, s) : launch2p_oct<N1, 0>(A, oct, s);
+    } else {
+        switch (oct & 3) {
+        case 0: return oct < 8 ? launch2<N1, 0, 0>(A, s) : launch2<N1, 0, 8>(A, s);
+        case 1: return oct < 8 ? launch2<N1, 0, 1>(A, s) : launch2<N1, 0, 8>(A, s);
+        case 2: return oct < 8 ? launch2<N1, 0, 2>(A, s) : launch2<N1, 0, 8>(A, s);
+        default: return oct < 8 ? launch2<N1, 0, 3>(A, s) : launch2<N1, 0, 8>(A, s);
+        }
     }
 }
 
