@@ -30,6 +30,7 @@ cudaError_t launch_stage1d_batch(int n1, const StageArgs *d_args, const int2 *d_
                                  int ctas, cudaStream_t s);
 cudaError_t set_batch_ops(int n1, const Ops &op);
 int stage1d_tasks(const StageArgs &A);
+int stage1d_batch_tasks(const StageArgs &A);
 int stage1d_batch_ctas(int n1);
 cudaError_t launch_init_maxwellian(float *f, const double *prim, const float *mi, const float *gmask, int nslots,
                                    int nvt, int E, int NP, const int n[3], const double v0[3], const double dv[3],
@@ -1960,7 +1961,7 @@ int batch_upload(bgk_batch *b, const double *dt)
         NewtonArgs N = newton_args(c, 0);
         N.err = b->err;
         na[q] = N;
-        const int64_t t = ts[q] + (int64_t)stage1d_tasks(sa[q]);
+        const int64_t t = ts[q] + (int64_t)stage1d_batch_tasks(sa[q]);
         const int64_t pt = ps[q] + c->npts;
         if (t > INT32_MAX / 2 || pt > INT32_MAX / 2)
             return bfail(b, BGK_EINVAL, "batch too large");
