@@ -954,16 +954,21 @@ int bgk_create(const bgk_mesh *mesh, int p, const bgk_vgrid *vg, double tau, con
     // per pass); above the limit the octants' own kernels and the smaller memory win.
     const int64_t fA = (int64_t)c->nvt * E * c->NP * kWarp;
     c->merged = c->opts.chunks == 0 && c->chunks.size() > 1 && fA * c->esize <= kMergeBytes;
-    const int64_t pool = c->merged ? 2 * fA : (int64_t)(c->chunks.size() + 1) * c->chunk_floats;
     // memory check before any allocation
-    const int64_t need = (fA + pool) * c->esize +
-                         (int64_t)c->max_groups * 5 * c->npts * 4 + c->npts * (5 * 8 * 3 + kParamStride * 4) +
-                         (int64_t)c->nslots * 4 * 25 +
-                         (c->prec == BGK_FP64 ? c->npts * 8 * (c->nv[0] + c->nv[1] + c->nv[2]) : 0) +
-                         (c->has_exchange ? 2 * (int64_t)c->nvt * c->ne[1] * c->ne[2] * c->NP * kWarp * 4 : 0);
+    const int64_t tables = (int64_t)c->max_groups * 5 * c->npts * 4 + c->npts * (5 * 8 * 3 + kParamStride * 4) +
+                           (int64_t)c->nslots * 4 * 25 +
+                           (c->prec == BGK_FP64 ? c->npts * 8 * (c->nv[0] + c->nv[1] + c->nv[2]) : 0) +
+                           (c->has_exchange ? 2 * (int64_t)c->nvt * c->ne[1] * c->ne[2] * c->NP * kWarp * 4 : 0);
+    int64_t pool = c->merged ? 2 * fA : (int64_t)(c->chunks.size() + 1) * c->chunk_floats;
+    int64_t need = (fA + pool) * c->esize + tables;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess)
         return bail(BGK_ECUDA, "cudaMemGetInfo failed (no CUDA device?)");
+    if (c->merged && (double)need > 0.97 * (double)free_b) {  // the two full buffers do not fit: chunk by chunk
+        c->merged = false;
+        pool = (int64_t)(c->chunks.size() + 1) * c->chunk_floats;
+        need = (fA + pool) * c->esize + tables;
+    }
     if ((double)need > 0.97 * (double)free_b)
         return bail(BGK_ENOMEM, "configuration needs " + std::to_string(need >> 20) + " MiB, only " +
                                     std::to_string(free_b >> 20) + " MiB free");
