@@ -7,6 +7,7 @@
 // A warp owns one (element, run of tiles) task; lane l holds velocity l of the tile, so every
 // global load or store of one node is one coalesced 128-byte line.
 #pragma once
+#include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -169,10 +170,14 @@ struct NewtonArgs {
     double v0[3], dv[3];
     float v0h[3], v0l[3], dvh[3], dvl[3];  // v0 and dv as double-float pairs (hi + lo)
     int n[3];
+    // what index_to_moments and the exponent need of the grid alone, formed once on the host: the axes' centres
+    // gc, gc dv / 2, -log2(e) / 2 (dv / 2)^2, the sum of gc^2 and the cell volume of the axes that have a spacing
+    double gc[3], gcs[3], gq[3], gcc, vol;
     int vdim;              // velocity dimension m: 3, or 2 (no u_z, E = rho |U|^2 / 2 + rho theta)
 };
 
-// Axis d of the Newton solve's velocity grid: first node v0, spacing dv, n nodes (with the FP32 pairs).
+// Axis d (0, 1, 2 in this order) of the Newton solve's velocity grid: first node v0, spacing dv, n nodes (with the
+// FP32 pairs and the grid's constants).
 inline void newton_axis(NewtonArgs &N, int d, double v0, double dv, int n)
 {
     N.v0[d] = v0;
@@ -182,6 +187,11 @@ inline void newton_axis(NewtonArgs &N, int d, double v0, double dv, int n)
     N.v0l[d] = (float)(v0 - (double)N.v0h[d]);
     N.dvh[d] = (float)dv;
     N.dvl[d] = (float)(dv - (double)N.dvh[d]);
+    N.gc[d] = std::fma((double)(n - 1), 0.5 * dv, v0);
+    N.gcs[d] = N.gc[d] * (0.5 * dv);
+    N.gq[d] = -0.5 * 1.4426950408889634 * (0.25 * dv * dv);
+    N.gcc = d == 0 ? N.gc[0] * N.gc[0] : std::fma(N.gc[d], N.gc[d], N.gcc);
+    N.vol = d == 0 ? dv : (d == 2 && n == 1 ? N.vol : N.vol * dv);  // an axis with one node has unit weight
 }
 
 // FR reference operators in FP64 for the plain all-FP64 form (Sec. 2.1, Eqs. 7-9).
@@ -274,7 +284,8 @@ struct WallArgs {
 // (xi_d = c_d + s_d m_d, s_d = dv_d / 2), the kernels accumulate
 //   mu = sum_k W_k (1, m_x, m_y, m_z, r_x m_x^2 + r_y m_y^2 + r_z m_z^2) f_k,  r_d = (s_d / s_x)^2 in FP32,
 // whose weights are exact FP32 numbers (r_d = 1 on grids with one spacing), so the only FP32 error of
-// the moments is the summation's. index_to_moments turns mu into Q = sum_k w_k psi_k f_k (Eq. 2).
+// the moments is the summation's. The Newton kernel's index_to_moments turns mu
+// into Q = sum_k w_k psi_k f_k (Eq. 2).
 // Trapezoid end factor of index k on an axis of n nodes: 1/2 at both ends, 1 inside; 1 on an axis with
 // a single node (the absent u_z of the two-dimensional velocity space).
 __host__ __device__ inline double end_factor(int k, int n) { return n > 1 && (k == 0 || k == n - 1) ? 0.5 : 1.0; }
@@ -282,22 +293,6 @@ __host__ __device__ inline double end_factor(int k, int n) { return n > 1 && (k 
 __host__ __device__ inline float index_r(double dv_d, double dv_x)
 {
     return (float)((dv_d / dv_x) * (dv_d / dv_x));
-}
-
-__host__ __device__ inline void index_to_moments(const double (&mu)[5], const double v0[3], const double dv[3],
-                                                 const int n[3], double (&Q)[5])
-{
-    // cell volume of the axes that have a spacing (an axis with one node has unit weight)
-    const double V = dv[0] * dv[1] * (n[2] > 1 ? dv[2] : 1.0), s0 = 0.5 * dv[0];
-    double cs = 0.0, cm = 0.0;
-    Q[0] = V * mu[0];
-    for (int d = 0; d < 3; d++) {
-        const double sd = 0.5 * dv[d], cd = v0[d] + (n[d] - 1) * sd;
-        Q[1 + d] = V * (cd * mu[0] + sd * mu[1 + d]);
-        cs += cd * cd;
-        cm += cd * sd * mu[1 + d];
-    }
-    Q[4] = 0.5 * V * (cs * mu[0] + 2.0 * cm + s0 * s0 * mu[4]);
 }
 
 // Index of the face element of element (ec) on face direction d: the two other coordinates.

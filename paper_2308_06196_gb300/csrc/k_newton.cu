@@ -222,12 +222,54 @@ __device__ __forceinline__ void sums64(double ad, double beta, double c0, double
 struct dfl {
     float hi, lo;
 };
+
+// Conversions between FP32 and FP64 on the integer pipe, bit for bit the hardware's: each conversion
+// instruction, like every FP64 one, holds the FP64 pipe for 16 clocks per warp. With them, the grid's constants
+// and the tests of signs and infinities off that pipe a point has 146 FP64 instructions instead of 225 (pipe
+// 62 -> 46 % busy, 262,144 points 169.5 -> 153 us per launch). Values outside the ranges below take the
+// instructions.
+__device__ __forceinline__ double widen(float v)
+{
+    const unsigned u = __float_as_uint(v), m = u & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u)  // zero, subnormal, infinite or NaN
+        return m == 0 ? __hiloint2double((int)u, 0) : (double)v;
+    return __hiloint2double((int)(((m >> 3) + 0x38000000u) | (u & 0x80000000u)), (int)(u << 29));
+}
+// x = 2^(E - 1023) 1.m: the upper 23 bits of m with E - 896 as the exponent, and round to nearest, ties to even,
+// on the lower 29
+__device__ __forceinline__ unsigned round_bits(unsigned hi, unsigned lo, unsigned &carry)
+{
+    const unsigned t = __funnelshift_l(lo, hi, 3);
+    carry = ((lo & 0x1fffffffu) + 0x0fffffffu + (t & 1u)) >> 29;
+    return (t + 0x40000000u + carry) | (hi & 0x80000000u);  // (+ 2^30: - 896 2^23 modulo 2^32)
+}
+__device__ __forceinline__ float narrow(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    if ((hi & 0x7fffffffu) - 0x38100000u >= 0x47d00000u - 0x38100000u)  // |x| outside [2^-126, 2^126)
+        return __double2float_rn(x);
+    unsigned carry;
+    return __uint_as_float(round_bits(hi, lo, carry));
+}
+// hi = the nearest FP32 number, lo = that of the rest: the rest is an integer of at most 29 bits times 2^(E - 1075)
 __device__ __forceinline__ dfl df_from(double x)
 {
-    const float h = __double2float_rn(x);
-    return {h, __double2float_rn(x - (double)h)};
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    if ((hi & 0x7fffffffu) - 0x3c300000u >= 0x47d00000u - 0x3c300000u) {  // |x| outside [2^-60, 2^126)
+        if (x == 0.0)
+            return {0.f, 0.f};
+        const float h = __double2float_rn(x);
+        return {h, __double2float_rn(x - (double)h)};
+    }
+    unsigned carry;
+    const unsigned h = round_bits(hi, lo, carry);
+    const float ulp = __uint_as_float((((hi << 3) & 0xff800000u) + 0x26000000u) | (hi & 0x80000000u));  // E - 948
+    return {__uint_as_float(h), (float)((int)(lo & 0x1fffffffu) - (int)(carry << 29)) * ulp};
 }
-__device__ __forceinline__ double df_val(dfl a) { return (double)a.hi + (double)a.lo; }
+__device__ __forceinline__ double df_val(dfl a) { return widen(a.hi) + widen(a.lo); }
+// x > 0 and x < infinity on the bits
+__device__ __forceinline__ bool finite64(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool positive64(double x) { return __double_as_longlong(x) > 0 && finite64(x); }
 __device__ __forceinline__ dfl df_mul(dfl a, dfl b)
 {
     const float p = __fmul_rn(a.hi, b.hi);
@@ -276,8 +318,8 @@ __device__ __forceinline__ dfl df_div(dfl a, dfl b)
 // |r| <= ln 2 / 2: ln 2 in three FP32 parts, the first with 12 significant bits so that n ln2_1 and
 // x - n ln2_1 are exact; e^r by its Taylor series to degree 11 (truncation below 1e-15 at |r| = 0.35),
 // Horner in double-float with the coefficients 1/k! as FP32 pairs; the result scaled by 2^n. Larger
-// arguments take the FP64 exponential.
-__device__ __forceinline__ dfl df_exp(dfl x)
+// arguments take the FP64 exponential. One copy for all its calls (see sums_dd_call).
+__device__ __noinline__ dfl df_exp(dfl x)
 {
     if (!(fabsf(x.hi) <= 10.f))
         return df_from(exp((double)x.hi + (double)x.lo));
@@ -308,13 +350,19 @@ __device__ __forceinline__ dfl df_exp(dfl x)
 // spacing); the first ratio exp(q1 + q2 (2 kp + 1)) is one exponential per axis; the downward ratio
 // E2 / rp a division. Relative error about 1e-13, far below what one refinement with the FP32 Jacobian
 // needs.
-__device__ __forceinline__ dfl sums_dd(dfl ad, dfl beta, dfl c0, dfl h, int n, dfl dv, dfl E2, dfl (&S)[3])
+struct SumsDd {
+    dfl lnp, S[3];
+};
+__device__ __forceinline__ SumsDd sums_dd(dfl ad, dfl beta, dfl c0, dfl h, int n, dfl dv, dfl E2)
 {
+    SumsDd o;
+    dfl(&S)[3] = o.S;
     if (n == 1) {  // one node of unit weight (no u_z, m = 2)
         S[0] = {1.f, 0.f};
         S[1] = c0;
         S[2] = df_mul(c0, c0);
-        return df_mul(c0, df_sub(ad, df_mulf(df_mul(beta, c0), 0.5f)));
+        o.lnp = df_mul(c0, df_sub(ad, df_mulf(df_mul(beta, c0), 0.5f)));
+        return o;
     }
     const dfl q1 = df_mul(df_sub(ad, df_mul(beta, c0)), h);
     const dfl q2 = df_mulf(df_mul(beta, df_mul(h, h)), -0.5f);
@@ -357,7 +405,25 @@ __device__ __forceinline__ dfl sums_dd(dfl ad, dfl beta, dfl c0, dfl h, int n, d
     S[0] = df_mul(df_sub(s0, df_scale(df_add(A0, Aend), 0.5f)), dv);
     S[1] = df_mul(df_sub(s1, df_scale(df_add(xa0, xae), 0.5f)), dv);
     S[2] = df_mul(df_sub(s2, df_scale(df_add(df_mul(c0e, xa0), df_mul(cend, xae)), 0.5f)), dv);
-    return df_mul(cp, df_sub(ad, df_mulf(df_mul(beta, cp), 0.5f)));
+    o.lnp = df_mul(cp, df_sub(ad, df_mulf(df_mul(beta, cp), 0.5f)));
+    return o;
+}
+
+// The one-lane form's three axes call one copy: inlined, the solve is larger than the instruction caches, and a
+// launch is held by its fetches (with df_exp, also one copy: 20,160 points 120 -> 80 us per launch, 262,144 points
+// 153 -> 147; the four-lane form has one axis per lane and is 2 us faster with its sums inlined).
+__device__ __noinline__ SumsDd sums_dd_call(dfl ad, dfl beta, dfl c0, dfl h, int n, dfl dv, dfl E2)
+{
+    return sums_dd(ad, beta, c0, h, n, dv, E2);
+}
+struct Sums64 {
+    double S[5];
+};
+__device__ __noinline__ Sums64 sums64_call(double ad, double beta, double c0, double h, int n, double dv)
+{
+    Sums64 o;
+    sums64<5>(ad, beta, c0, h, n, dv, o.S);
+    return o;
 }
 
 // The moments M[g psi~] (5) of assemble() from double-float 1-D sums S[d][0..2], scaled by e0.
@@ -370,6 +436,20 @@ __device__ __forceinline__ void assemble_dd(const dfl (&S)[3][3], dfl e0, dfl (&
         M[1 + d] = df_mul(e0, df_mul(S[d][1], o0[d]));
     const dfl m4 = df_add(df_add(df_mul(S[0][2], o0[0]), df_mul(S[1][2], o0[1])), df_mul(S[2][2], o0[2]));
     M[4] = df_mul(e0, df_scale(m4, 0.5f));
+}
+
+// Q from the grid-index moments mu (the weights' note in bgk_common.cuh)
+__device__ __forceinline__ void index_to_moments(const NewtonArgs &A, const double (&mu)[5], double (&Q)[5])
+{
+    const double s0 = 0.5 * A.dv[0];
+    double cm = 0.0;
+    Q[0] = A.vol * mu[0];
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        Q[1 + d] = A.vol * fma(0.5 * A.dv[d], mu[1 + d], A.gc[d] * mu[0]);
+        cm += A.gcs[d] * mu[1 + d];
+    }
+    Q[4] = 0.5 * A.vol * (A.gcc * mu[0] + 2.0 * cm + s0 * s0 * mu[4]);
 }
 
 // The solve of one point by L = 1 or 4 lanes. With L = 4 the lanes d = 0, 1, 2 of a point's group form the
@@ -433,16 +513,16 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
             const float h0 = hi[0], l0 = lo[0], h4 = hi[1], l4 = lo[1];
 #pragma unroll
             for (int c = 0; c < 5; c++)
-                Q[c] = (double)from(c < 4 ? h0 : h4, c & 3) + (double)from(c < 4 ? l0 : l4, c & 3);
+                Q[c] = df_val({from(c < 4 ? h0 : h4, c & 3), from(c < 4 ? l0 : l4, c & 3)});
         } else {
 #pragma unroll
             for (int c = 0; c < 5; c++)
-                Q[c] = (double)hi[c % kC] + (double)lo[c % kC];
+                Q[c] = df_val({hi[c % kC], lo[c % kC]});
         }
     }
     if (!A.Qin) {  // the FP32 kernels sum in the grid-index basis
         const double mu[5] = {Q[0], Q[1], Q[2], Q[3], Q[4]};
-        index_to_moments(mu, A.v0, A.dv, A.n, Q);
+        index_to_moments(A, mu, Q);
     }
     if (writer)
 #pragma unroll
@@ -454,7 +534,7 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
     const double hm = 0.5 * A.vdim;  // E = rho |U|^2 / 2 + (m / 2) rho theta
     const double thc = (Q[4] * irho - 0.5 * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2])) * (A.vdim == 2 ? 1.0 : 2.0 / 3.0);
     float *par = A.param + (int64_t)pt * kParamStride;
-    if (!(rho > 0.0) || !(thc > 0.0) || !isfinite(rho) || !isfinite(thc)) {
+    if (!positive64(rho) || !positive64(thc)) {
         if (!writer)
             return;
         atomicOr(A.err, kErrDomain);
@@ -474,7 +554,8 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
     double lnc0 = 0.0;  // warm start in the lnC form: alpha_0 of the centred basis directly
     if (!A.cold && !A.continuous) {
         const double *pp = A.prim + (int64_t)pt * 5;
-        if ((A.lnc_form || pp[0] > 0.0) && pp[4] > 0.0 && isfinite(pp[0] + pp[1] + pp[2] + pp[3] + pp[4])) {
+        if ((A.lnc_form ? finite64(pp[0]) : positive64(pp[0])) && positive64(pp[4]) && finite64(pp[1]) &&
+            finite64(pp[2]) && finite64(pp[3])) {
             rh0 = pp[0];
             lnc0 = pp[0];
             V[0] = pp[1];
@@ -508,7 +589,7 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
     }
 
     // the ablation (continuous Maxwellian of Q) stops here: alpha = the starting state itself
-    double corr = 0.0;
+    float corr = 0.f;
     if (!A.continuous) {
         // FP32 Newton iterations until the step is below FP32 resolution (it32 minimum, 30 maximum), all
         // in FP32: the steps accumulate in da and are added to the FP64 alpha once at the end
@@ -611,19 +692,23 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
                                 ? E2[d - 1]
                                 : df_exp(df_mul(ald[4], df_mul(hd[d], hd[d])));
     #pragma unroll
-                for (int d = 0; d < 3; d++)
-                    lnp = df_add(lnp, sums_dd(ald[1 + d], beta, c0d[d], hd[d], A.n[d], dvd[d], E2[d], S[d]));
+                for (int d = 0; d < 3; d++) {
+                    const SumsDd o = sums_dd_call(ald[1 + d], beta, c0d[d], hd[d], A.n[d], dvd[d], E2[d]);
+                    lnp = df_add(lnp, o.lnp);
+    #pragma unroll
+                    for (int m = 0; m < 3; m++)
+                        S[d][m] = o.S[m];
+                }
             } else {  // lane 3 repeats axis 2
-                dfl So[3];
                 const dfl ho = pick(hd[0], hd[1], hd[2]);
-                const dfl lo = sums_dd(pick(ald[1], ald[2], ald[3]), beta, pick(c0d[0], c0d[1], c0d[2]), ho, nax,
-                                       pick(dvd[0], dvd[1], dvd[2]), df_exp(df_mul(ald[4], df_mul(ho, ho))), So);
+                const SumsDd o = sums_dd(pick(ald[1], ald[2], ald[3]), beta, pick(c0d[0], c0d[1], c0d[2]), ho, nax,
+                                         pick(dvd[0], dvd[1], dvd[2]), df_exp(df_mul(ald[4], df_mul(ho, ho))));
     #pragma unroll
                 for (int d = 0; d < 3; d++) {
     #pragma unroll
                     for (int m = 0; m < 3; m++)
-                        S[d][m] = {from(So[m].hi, d), from(So[m].lo, d)};
-                    lnp = df_add(lnp, {from(lo.hi, d), from(lo.lo, d)});
+                        S[d][m] = {from(o.S[m].hi, d), from(o.S[m].lo, d)};
+                    lnp = df_add(lnp, {from(o.lnp.hi, d), from(o.lnp.lo, d)});
                 }
             }
             dfl M[5];
@@ -663,7 +748,8 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
             al[m] = df_val(ald[m]);
     }
     const double beta = -al[4];
-    if (!(beta > 0.0) || !isfinite(al[0] + al[1] + al[2] + al[3]) || corr >= 1e-6) {
+    if (!positive64(beta) || !finite64(al[0]) || !finite64(al[1]) || !finite64(al[2]) || !finite64(al[3]) ||
+        corr > 1e-6f) {  // (1e-6f is the largest FP32 number below 1e-6)
         if (writer)
             atomicOr(A.err, kErrNewton);
         return;
@@ -674,8 +760,12 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
     if (force) {
         if constexpr (L == 1) {
 #pragma unroll
-            for (int d = 0; d < 3; d++)
-                sums64<5>(al[1 + d], -al[4], df_val(c0d[d]), df_val(hd[d]), A.n[d], A.dv[d], Sf[d]);
+            for (int d = 0; d < 3; d++) {
+                const Sums64 o = sums64_call(al[1 + d], -al[4], df_val(c0d[d]), df_val(hd[d]), A.n[d], A.dv[d]);
+#pragma unroll
+                for (int m = 0; m < 5; m++)
+                    Sf[d][m] = o.S[m];
+            }
         } else {
             auto axis = [&](auto x, auto y, auto z) { return sub == 0 ? x : (sub == 1 ? y : z); };
             const dfl c0 = axis(c0d[0], c0d[1], c0d[2]), h = axis(hd[0], hd[1], hd[2]);
@@ -720,24 +810,23 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
     double e2 = 0.0;
     for (int d = 0; d < 3; d++) {
         const double sd = 0.5 * A.dv[d];
-        const double ed = A.v0[d] + (A.n[d] - 1) * sd - Up[d];
+        const double ed = A.gc[d] - Up[d];
         e2 += ed * ed;
-        par[1 + d] = (float)(-L2E * ed * sd * it2);
+        par[1 + d] = narrow(-L2E * ed * sd * it2);
     }
     const double Aexp = L2E * (lnC - 0.5 * e2 * it2);
     const double j = fmin(20.0, fmax(-20.0, rint(Aexp)));
-    par[0] = (float)(Aexp - j);
+    par[0] = narrow(Aexp - j);
     if (A.dv[0] == A.dv[1] && A.dv[0] == A.dv[2]) {
-        const double q = -0.5 * L2E * (0.25 * A.dv[0] * A.dv[0]) * it2;
-        const float qh = (float)q;
-        par[4] = qh;
-        par[5] = (float)(q - (double)qh);
+        const dfl q = df_from(A.gq[0] * it2);
+        par[4] = q.hi;
+        par[5] = q.lo;
         par[6] = 0.f;
     } else {
         for (int d = 0; d < 3; d++)
-            par[4 + d] = (float)(-0.5 * L2E * (0.25 * A.dv[d] * A.dv[d]) * it2);
+            par[4 + d] = narrow(A.gq[d] * it2);
     }
-    par[7] = kExp2Magic + (float)j;
+    par[7] = kExp2Magic + narrow(j);
     if (A.mu_ref > 0.0) {  // variable collision time of this point's state: 1/tau = rho theta / mu(theta)
         const double itau = rho * thc / (A.mu_ref * pow(thc, A.mu_omega));
         par[6] = (float)itau;
@@ -787,15 +876,14 @@ __device__ __forceinline__ void newton_point(const NewtonArgs &A, const int pt)
 // The two forms of the solve, by the number of points (128-thread CTAs on 152 SMs; us per launch alone,
 // before -> now, with the partial sums' loads four groups at a time):
 //   up to 9,728    latency: four lanes share a point, 4 CTAs per SM leave the 128 registers that avoid
-//                  spills (72 points 44 -> 23; 6,000 points 80 -> 39). Up to 19,456 points (one wave) the launch
+//                  spills (72 points 44 -> 22; 6,000 points 80 -> 39). Up to 19,456 points (one wave) the launch
 //                  itself is still shorter (12,000 points 90 -> 47), but the FP64 set-up that the four lanes
 //                  repeat costs other work on the SMs more (13,440 points, three contexts in turn 5.57
 //                  against 5.49 ms per pass);
-//   beyond         the FP64 pipe (a warp instruction per 16 clocks and SM; some 230 per point in the set-up
-//                  and the outputs) and the chains' latency: a thread per point, 8 CTAs (64 registers,
-//                  spilling to L1) keep it busiest (262,144 points 170 -> 164; 4 CTAs 198, four lanes per
-//                  point 512; 20,160 points 99 alone with 4 CTAs against 107, but three contexts in turn 5.59
-//                  against 5.42 ms per pass).
+//   beyond         issue (61 % of the cycles), the FP64 pipe (46 %; a warp instruction per 16 clocks and SM, 146 per
+//                  point in the set-up and the outputs) and the chains' latency: a thread per point, 6 CTAs (80
+//                  registers, the rest spilled to L1) keep them busiest (262,144 points 147; 8 CTAs 153, 5
+//                  CTAs 149, four lanes per point 512; 20,160 points 80 each).
 // With a body force the set-up is longer and the limit two thirds of that (9,720 points, three contexts in turn:
 // 6.96 against 6.87 ms per pass).
 // The batched solve, whose arguments come from global memory, runs best at 4 CTAs.
@@ -847,7 +935,7 @@ cudaError_t launch_newton(const NewtonArgs &A, cudaStream_t s)
     if (A.npts <= (force ? kLanePoints * 2 / 3 : kLanePoints))
         k_newton<4, 4><<<newton_ctas(A.npts, 4), kNewtonThreads, 0, s>>>(A);
     else
-        k_newton<1, 8><<<newton_ctas(A.npts, 1), kNewtonThreads, 0, s>>>(A);
+        k_newton<1, 6><<<newton_ctas(A.npts, 1), kNewtonThreads, 0, s>>>(A);
     return cudaGetLastError();
 }
 
