@@ -200,6 +200,7 @@ struct bgk_ctx {
     std::vector<unsigned char> toct_h;  // sign octant of every tile
     std::vector<Chunk> chunks;
     int64_t chunk_floats = 0;  // floats per pool slot
+    bool task_fixed = false;   // G is the task length too (chosen by the user or the autotuner)
     bool merged = false;       // small problem: one launch per stage over all chunks, two full stage buffers
     // device buffers
     float *fA = nullptr, *pool = nullptr;
@@ -323,6 +324,7 @@ StageArgs stage_args(bgk_ctx *c, const Chunk &ch)
     A.vt0 = ch.vt0;
     A.nvt = ch.nvt;
     A.G = c->G;
+    A.fixed = c->task_fixed;
     A.group0 = ch.group0;
     A.ngroups = A.ntasks = ch.ngroups;
     A.R = 1;
@@ -921,7 +923,7 @@ int bgk_create(const bgk_mesh *mesh, int p, const bgk_vgrid *vg, double tau, con
         maxc = std::max(maxc, ch.nvt);
     // tiles per warp task: enough tasks for ~32 resident warps per SM, at most 8 tiles
     if (c->opts.vtiles_per_task > 0)
-        c->G = c->opts.vtiles_per_task;
+        c->G = c->opts.vtiles_per_task, c->task_fixed = true;
     else {
         const int64_t tasks1 = (int64_t)maxc * E;
         c->G = (int)std::max<int64_t>(1, std::min<int64_t>(8, tasks1 / (152 * 32)));
@@ -1772,6 +1774,7 @@ static std::vector<int> task_length_candidates(int maxc)
 static void set_task_length(bgk_ctx *c, int G)
 {
     c->G = G;
+    c->task_fixed = true;
     c->ngroups = 0;
     for (auto &ch : c->chunks) {
         ch.group0 = c->ngroups;
@@ -1954,7 +1957,7 @@ int batch_upload(bgk_batch *b, const double *dt)
             real += c->slotk[v] >= 0;
         for (int st = 0; st < 3; st++) {
             StageArgs A = stage_args(c, ch);
-            A.R = std::max(1, kBatchTiles / A.G);
+            A.R = A.fixed ? 1 : std::max(1, kBatchTiles / A.G);
             A.ntasks = (A.ngroups + A.R - 1) / A.R;
             A.src = st == 0 ? Aq : (st == 1 ? s1 : s2);
             A.fn = st == 0 ? nullptr : Aq;

@@ -76,6 +76,7 @@ struct StageArgs {
     int vt0;             // first global tile of the chunk
     int nvt;             // tiles in the chunk
     int G;               // tiles per moment group
+    int fixed;           // 1: G was chosen by the user or the autotuner and is the task's length too
     int R, ntasks;       // moment groups per task, tasks per element (plan_tasks)
     int group0;          // global index of the launch's first moment group
     int ngroups;         // moment groups of the launch
@@ -124,7 +125,10 @@ inline void plan_tasks(StageArgs &A, int64_t units, int64_t wave, double start, 
 {
     A.R = 1;
     A.ntasks = A.ngroups;
-    if (A.nseg > 1)  // (several chunks in a small problem's launch: the groups as they are)
+    // A length that the user gave or the autotuner measured is the task's: the rule knows nothing of the reuse of
+    // neighbours in L2 (128 x 8 x 8 elements of 48^3 velocities at p = 2: 7.97 ms per launch with the rule on the
+    // autotuner's candidates, 7.48 with its own pick). So are the groups of several chunks in one launch.
+    if (A.nseg > 1 || A.fixed)
         return;
     auto last = [&](double x) { return x > 0.0 ? idle + (1.0 - idle) * x : 0.0; };
     double best = 0.0;

@@ -20,7 +20,7 @@ namespace bgk {
 // Every copy has a role lane (operand and half) that announces and issues its bytes on the buffer's barrier.
 // Bound: latency and issue at 12 warps per SM. With a lane per velocity (k_stage2) the exponents alone returned
 // 8 of the 24 cycles of shared-memory data per 32 degrees of freedom, and the neighbour lines came from L2
-// lane by lane: 128^2 elements at p = 3, 32^2 velocities 0.174 -> 0.151 ms per octant launch (4.7 TB/s); 128 x
+// lane by lane: 128^2 elements at p = 3, 32^2 velocities 0.174 -> 0.154 ms per octant launch (4.6 TB/s); 128 x
 // 127 at p = 1, 40^2 velocities, three steps 5.72 -> 3.75 ms.
 // Forms: GEN = 0 every face periodic, no limiter, constant tau, one velocity spacing; GEN = 1 everything.
 // ------------------------------------------------------------------------------------------------

@@ -1,6 +1,6 @@
 // k_stage3c.cuh -- the fused SSP-RK3 stage kernel of curvilinear hexahedra on the structured element
-// grid (FP32-split form), every operand staged in shared memory by bulk asynchronous copies as in
-// k_stage3s.cuh; instantiated per degree in k_stage3_p*.cu.
+// grid (FP32-split form), every operand staged in shared memory by bulk asynchronous copies; instantiated
+// per degree in k_stage3_p*.cu.
 #pragma once
 #include <type_traits>
 
@@ -15,8 +15,8 @@ namespace bgk {
 // ------------------------------------------------------------------------------------------------
 // Curvilinear hexahedra, structured element grid (Sec. 2.1, Eqs. 6-9 on the mapped element): the
 // reference-space flux u f with u = Ja^d . xi at every node, and the upwind common flux of every face
-// point from the sign of the shared face normal's N . xi per lane. The layout and the copy schedule are
-// k_stage3s's: one CTA per (element, run of G velocity tiles), one warp per z-layer, lane = velocity of
+// point from the sign of the shared face normal's N . xi per lane. Layout and
+// copy schedule: one CTA per (element, run of G velocity tiles), one warp per z-layer, lane = velocity of
 // the tile; the warp's f_s layer double-buffered, three rotating slots per warp for f^n and the upwind
 // neighbours' layers, the velocity tables double-buffered by warp 0. The staged neighbour of direction
 // d is the one on the side the tile's sign octant makes upwind (the low side where xi_d >= 0): a face
@@ -30,7 +30,7 @@ struct Stage3cSmem {
     float fs[2][NP][kWarp];
     float sl[N1][3][NQ][kWarp];
     float tab[2][kTabRows][kWarp];
-    float par[N1][(NQ + 1) / 2][kParamStride][2];  // BGK exponents by layer and node pair (see k_stage3s)
+    float par[N1][(NQ + 1) / 2][kParamStride][2];  // BGK exponents by layer and node pair
     float fpar[GEN ? NP : 1][GEN ? kParamStride : 4];
     float lim[GEN ? 2 : 1][GEN ? N1 : 1][GEN ? kWarp : 4];
     float4 met[NP][3];      // metric rows Ja^d; .w of row 0 = -b dt / J (the line sums' factor), of row 1 = W J
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(kWarp *N1, (N1 >= 4 ? BGK_STAGE3C_MINCTAS_P3 :
         for (int d = 0; d < 3; d++)
             en[d] = upwind_neighbour(A.mesh, ec, d, ((oct >> d) & 1) != 0);
     };
-    // role lanes as in k_stage3s: lane 0 the f_s layer, RZ .. RZ + N1 - 1 the z-neighbour's row groups,
+    // role lanes: lane 0 the f_s layer, RZ .. RZ + N1 - 1 the z-neighbour's row groups,
     // RFN the f^n layer, RX / RY the x- / y-neighbour's layer w, RT of warp 0 the velocity table
     constexpr int RZ = 1, RFN = N1 + 1, RX = N1 + 2, RY = N1 + 3, RT = N1 + 4;
     const int64_t tstride = (int64_t)E * NP * kWarp;

@@ -26,7 +26,7 @@ namespace bgk {
 // Shared memory per warp (bulk copies, the warp's own mbarriers):
 //   fs     f_s of the element: read into registers at the start of the tile, after which the next
 //          tile's f_s lands there;
-//   sl[3]  three rotating slots of one element each, as k_stage3s: at tile t slot t mod 3 holds f^n,
+//   sl[3]  three rotating slots of one element each: at tile t slot t mod 3 holds f^n,
 //          slot t+1 the x-upwind neighbour and slot t+2 the y-upwind neighbour; slot t mod 3 then takes
 //          the z-upwind neighbour (read by the z-lines), then the tile's output, transposed, for the
 //          moment sums; each slot takes the next tile's copies as soon as it is consumed;
