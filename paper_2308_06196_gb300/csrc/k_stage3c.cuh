@@ -252,437 +252,438 @@ __global__ void __launch_bounds__(kWarp *N1, (N1 >= 4 ? BGK_STAGE3C_MINCTAS_P3 :
     const float kb = A.kb;
 
     int ka = 0;
-    for (int vl = vl0; vl < vl1; vl++) {
-        const int vt = A.vt0 + vl;
-        const int slot = vt * kWarp + lane;
-        const int b = (vl - vl0) & 1;
-        const int kx = ka == 2 ? 0 : ka + 1, ky = ka == 0 ? 2 : ka - 1;
-        int enn[3] = {en[0], en[1], en[2]};
-        const bool more = vl + 1 < vl1;
-        const int octn = more ? (int)__ldg(A.toct + vt + 1) : octc;
-        const bool turn = octn != octc;  // the next tile lies in another octant
-        if (turn)
-            nbrs_oct(octn, enn);
-        __syncwarp();
-        if (lane == 0 && more) {
-            fence_proxy_async();
-            mbar_arrive_expect_tx(bar(b ^ 1), kSlot);
-            bulk_g2s(fs0 + (b ^ 1) * kFsBuf, fsrc + (vl + 1) * tstride, kSlot, bar(b ^ 1));
-        }
-        const int oct = octc;
-        const bool l0 = (oct & 1) != 0, l1 = (oct & 2) != 0, l2 = (oct & 4) != 0;
-        const int enx = en[0], eny = en[1], enz = en[2];
-
-        wait(b);
-        mbar_wait(tbar(b), (ph >> (5 + b)) & 1, A.err);
-        ph ^= 1u << (5 + b);
-        const float m0 = sm.tab[b][0][lane], m1 = sm.tab[b][1][lane], m2 = sm.tab[b][2][lane];
-        const float x0 = fmaf(A.vs[0], m0, A.vc[0]), x1 = fmaf(A.vs[1], m1, A.vc[1]), x2 = fmaf(A.vs[2], m2, A.vc[2]);
-        float acc[NQ];
-        if (has_fn) {
-            wait(2 + ka);
-#pragma unroll
-            for (int q = 0; q < NQ; q++)
-                acc[q] = sm.sl[w][ka][q][lane];
-        } else {
-#pragma unroll
-            for (int q = 0; q < NQ; q++)
-                acc[q] = 0.f;
-        }
-        // slot ka is consumed: the z-neighbour's slice lands there
-        __syncwarp();
-        if (lane >= RZ && lane < RZ + N1) {
-            const float *zs = csrc;
-            const uint32_t bb = bar(2 + ka);
-            fence_proxy_async();
-            if (lane == RZ)
-                mbar_arrive_expect_tx(bb, zs ? kSlot : 0);
-            if (zs)
-                bulk_g2s(sl0 + ka * kSlot + (lane - RZ) * N1 * kRow, zs + vl * tstride, N1 * kRow, bb);
-        }
-        // (launch-uniform feature tests sit outside the unrolled node loops, which stay one basic block)
-        if (GEN && A.vtau) {
-#pragma unroll
-            for (int q = 0; q < NQ; q++)
-                acc[q] = fmaf(A.an, acc[q],
-                              __fsub_rn(A.b, __fmul_rn(bdt, sm.par[w][q / 2][6][q % 2])) * sm.fs[b][q + NQ * w][lane]);
-        } else {
-#pragma unroll
-            for (int q = 0; q < NQ; q++)
-                acc[q] = fmaf(A.an, acc[q], kb * sm.fs[b][q + NQ * w][lane]);
-        }
-        // The lines of direction d through this warp's nodes: x- and y-lines of layer w (their sums
-        // go to acc), z-lines of slice w (their sums overwrite the rows they read, after B1). Line ln
-        // has face point fp = ln + N1 w on both faces. lo: the tile's octant stages the low-side
-        // neighbour (slot ks); es: that neighbour, < 0 on a boundary face (its ghost value instead).
-        // Lanes whose flow enters through the other face take that face's exterior trace, read for all
-        // lines of the direction at once and only where some lane of the warp needs it.
-        auto lines = [&](auto dc, int ks, bool lo, int es) {
-            constexpr int d = decltype(dc)::value;
-            auto node = [&](int ln, int j) {  // element node j of line ln
-                return d == 0 ? j + N1 * ln + NQ * w : (d == 1 ? ln + N1 * j + NQ * w : ln + N1 * w + NQ * j);
-            };
-            auto srow = [&](int ln, int j) { return d == 0 ? j + N1 * ln : ln + N1 * j; };  // row in slot ks
-            float cS[N1], cF[N1];  // trace weights of the staged and of the other side's neighbour
-#pragma unroll
-            for (int j = 0; j < N1; j++) {
-                cS[j] = lo ? A.ops.lp[j] : A.ops.lm[j];
-                cF[j] = lo ? A.ops.lm[j] : A.ops.lp[j];
+    for (int vl = vl0; vl < vl1;) {  // a moment group
+        for (; vl < ge; vl++) {
+            const int vt = A.vt0 + vl;
+            const int slot = vt * kWarp + lane;
+            const int b = (vl - vl0) & 1;
+            const int kx = ka == 2 ? 0 : ka + 1, ky = ka == 0 ? 2 : ka - 1;
+            int enn[3] = {en[0], en[1], en[2]};
+            const bool more = vl + 1 < vl1;
+            const int octn = more ? (int)__ldg(A.toct + vt + 1) : octc;
+            const bool turn = octn != octc;  // the next tile lies in another octant
+            if (turn)
+                nbrs_oct(octn, enn);
+            __syncwarp();
+            if (lane == 0 && more) {
+                fence_proxy_async();
+                mbar_arrive_expect_tx(bar(b ^ 1), kSlot);
+                bulk_g2s(fs0 + (b ^ 1) * kFsBuf, fsrc + (vl + 1) * tstride, kSlot, bar(b ^ 1));
             }
-            auto trace = [&](const float(&v)[N1], const float(&c)[N1]) {  // trace_line with weights c
-                float t = 0.f;
+            const int oct = octc;
+            const bool l0 = (oct & 1) != 0, l1 = (oct & 2) != 0, l2 = (oct & 4) != 0;
+            const int enx = en[0], eny = en[1], enz = en[2];
+
+            wait(b);
+            mbar_wait(tbar(b), (ph >> (5 + b)) & 1, A.err);
+            ph ^= 1u << (5 + b);
+            const float m0 = sm.tab[b][0][lane], m1 = sm.tab[b][1][lane], m2 = sm.tab[b][2][lane];
+            const float x0 = fmaf(A.vs[0], m0, A.vc[0]), x1 = fmaf(A.vs[1], m1, A.vc[1]), x2 = fmaf(A.vs[2], m2, A.vc[2]);
+            float acc[NQ];
+            if (has_fn) {
+                wait(2 + ka);
 #pragma unroll
-                for (int j = 1; j < N1; j++)
-                    t = fmaf(c[j], v[j] - v[0], t);
-                return v[0] + t;
-            };
-            float uL[N1], uR[N1], tF[N1];
-            bool far = false;
-            if constexpr (N1 % 2 == 0) {  // two face points at a time (the same operations per half)
-                const unsigned long long X0 = pack2(x0, x0), X1 = pack2(x1, x1), X2 = pack2(x2, x2);
-#pragma unroll
-                for (int ln = 0; ln < N1; ln += 2) {
-                    const int pr = (ln + N1 * w) / 2;
-                    float u2[2][2];
-#pragma unroll
-                    for (int sd = 0; sd < 2; sd++) {
-                        const float4 n0 = sm.fnmp[d][sd][pr][0], n1 = sm.fnmp[d][sd][pr][1];
-                        unpack2(ffma2(pack2(n1.x, n1.y), X2, ffma2(pack2(n0.z, n0.w), X1, fmul2(pack2(n0.x, n0.y), X0))),
-                                u2[sd][0], u2[sd][1]);
-                    }
-#pragma unroll
-                    for (int h = 0; h < 2; h++) {
-                        uL[ln + h] = u2[0][h];
-                        uR[ln + h] = u2[1][h];
-                        tF[ln + h] = 0.f;
-                        far = far || (lo ? uR[ln + h] < 0.f : uL[ln + h] > 0.f);
-                    }
-                }
+                for (int q = 0; q < NQ; q++)
+                    acc[q] = sm.sl[w][ka][q][lane];
             } else {
 #pragma unroll
-                for (int ln = 0; ln < N1; ln++) {
-                    const int fp = ln + N1 * w;
-                    const float4 nL = sm.fnm[d][0][fp], nR = sm.fnm[d][1][fp];
-                    uL[ln] = fmaf(nL.z, x2, fmaf(nL.y, x1, nL.x * x0));
-                    uR[ln] = fmaf(nR.z, x2, fmaf(nR.y, x1, nR.x * x0));
-                    tF[ln] = 0.f;
-                    far = far || (lo ? uR[ln] < 0.f : uL[ln] > 0.f);
-                }
+                for (int q = 0; q < NQ; q++)
+                    acc[q] = 0.f;
             }
-            if (__any_sync(0xffffffffu, far)) {
-                const int g = 2 * d + (lo ? 1 : 0);
-                const int eo = upwind_neighbour(A.mesh, ec, d, !lo);
-                if (!GEN || eo >= 0) {
-                    const float *nb = A.src + fidx(vl, eo, 0, lane, E, NP);
-                    float v[N1][N1];
+            // slot ka is consumed: the z-neighbour's slice lands there
+            __syncwarp();
+            if (lane >= RZ && lane < RZ + N1) {
+                const float *zs = csrc;
+                const uint32_t bb = bar(2 + ka);
+                fence_proxy_async();
+                if (lane == RZ)
+                    mbar_arrive_expect_tx(bb, zs ? kSlot : 0);
+                if (zs)
+                    bulk_g2s(sl0 + ka * kSlot + (lane - RZ) * N1 * kRow, zs + vl * tstride, N1 * kRow, bb);
+            }
+            // (launch-uniform feature tests sit outside the unrolled node loops, which stay one basic block)
+            if (GEN && A.vtau) {
+#pragma unroll
+                for (int q = 0; q < NQ; q++)
+                    acc[q] = fmaf(A.an, acc[q],
+                                  __fsub_rn(A.b, __fmul_rn(bdt, sm.par[w][q / 2][6][q % 2])) * sm.fs[b][q + NQ * w][lane]);
+            } else {
+#pragma unroll
+                for (int q = 0; q < NQ; q++)
+                    acc[q] = fmaf(A.an, acc[q], kb * sm.fs[b][q + NQ * w][lane]);
+            }
+            // The lines of direction d through this warp's nodes: x- and y-lines of layer w (their sums
+            // go to acc), z-lines of slice w (their sums overwrite the rows they read, after B1). Line ln
+            // has face point fp = ln + N1 w on both faces. lo: the tile's octant stages the low-side
+            // neighbour (slot ks); es: that neighbour, < 0 on a boundary face (its ghost value instead).
+            // Lanes whose flow enters through the other face take that face's exterior trace, read for all
+            // lines of the direction at once and only where some lane of the warp needs it.
+            auto lines = [&](auto dc, int ks, bool lo, int es) {
+                constexpr int d = decltype(dc)::value;
+                auto node = [&](int ln, int j) {  // element node j of line ln
+                    return d == 0 ? j + N1 * ln + NQ * w : (d == 1 ? ln + N1 * j + NQ * w : ln + N1 * w + NQ * j);
+                };
+                auto srow = [&](int ln, int j) { return d == 0 ? j + N1 * ln : ln + N1 * j; };  // row in slot ks
+                float cS[N1], cF[N1];  // trace weights of the staged and of the other side's neighbour
+#pragma unroll
+                for (int j = 0; j < N1; j++) {
+                    cS[j] = lo ? A.ops.lp[j] : A.ops.lm[j];
+                    cF[j] = lo ? A.ops.lm[j] : A.ops.lp[j];
+                }
+                auto trace = [&](const float(&v)[N1], const float(&c)[N1]) {  // trace_line with weights c
+                    float t = 0.f;
+#pragma unroll
+                    for (int j = 1; j < N1; j++)
+                        t = fmaf(c[j], v[j] - v[0], t);
+                    return v[0] + t;
+                };
+                float uL[N1], uR[N1], tF[N1];
+                bool far = false;
+                if constexpr (N1 % 2 == 0) {  // two face points at a time (the same operations per half)
+                    const unsigned long long X0 = pack2(x0, x0), X1 = pack2(x1, x1), X2 = pack2(x2, x2);
+#pragma unroll
+                    for (int ln = 0; ln < N1; ln += 2) {
+                        const int pr = (ln + N1 * w) / 2;
+                        float u2[2][2];
+#pragma unroll
+                        for (int sd = 0; sd < 2; sd++) {
+                            const float4 n0 = sm.fnmp[d][sd][pr][0], n1 = sm.fnmp[d][sd][pr][1];
+                            unpack2(ffma2(pack2(n1.x, n1.y), X2, ffma2(pack2(n0.z, n0.w), X1, fmul2(pack2(n0.x, n0.y), X0))),
+                                    u2[sd][0], u2[sd][1]);
+                        }
+#pragma unroll
+                        for (int h = 0; h < 2; h++) {
+                            uL[ln + h] = u2[0][h];
+                            uR[ln + h] = u2[1][h];
+                            tF[ln + h] = 0.f;
+                            far = far || (lo ? uR[ln + h] < 0.f : uL[ln + h] > 0.f);
+                        }
+                    }
+                } else {
 #pragma unroll
                     for (int ln = 0; ln < N1; ln++) {
-                        const bool need = lo ? uR[ln] < 0.f : uL[ln] > 0.f;
-#pragma unroll
-                        for (int j = 0; j < N1; j++)
-                            v[ln][j] = need ? __ldg(nb + node(ln, j) * kWarp) : 0.f;
+                        const int fp = ln + N1 * w;
+                        const float4 nL = sm.fnm[d][0][fp], nR = sm.fnm[d][1][fp];
+                        uL[ln] = fmaf(nL.z, x2, fmaf(nL.y, x1, nL.x * x0));
+                        uR[ln] = fmaf(nR.z, x2, fmaf(nR.y, x1, nR.x * x0));
+                        tF[ln] = 0.f;
+                        far = far || (lo ? uR[ln] < 0.f : uL[ln] > 0.f);
                     }
+                }
+                if (__any_sync(0xffffffffu, far)) {
+                    const int g = 2 * d + (lo ? 1 : 0);
+                    const int eo = upwind_neighbour(A.mesh, ec, d, !lo);
+                    if (!GEN || eo >= 0) {
+                        const float *nb = A.src + fidx(vl, eo, 0, lane, E, NP);
+                        float v[N1][N1];
 #pragma unroll
-                    for (int ln = 0; ln < N1; ln++)
-                        tF[ln] = trace(v[ln], cF);
-                } else {
-                    // (the wall test is outside the loops: no load is formed from a pointer that may be null)
+                        for (int ln = 0; ln < N1; ln++) {
+                            const bool need = lo ? uR[ln] < 0.f : uL[ln] > 0.f;
+#pragma unroll
+                            for (int j = 0; j < N1; j++)
+                                v[ln][j] = need ? __ldg(nb + node(ln, j) * kWarp) : 0.f;
+                        }
+#pragma unroll
+                        for (int ln = 0; ln < N1; ln++)
+                            tF[ln] = trace(v[ln], cF);
+                    } else {
+                        // (the wall test is outside the loops: no load is formed from a pointer that may be null)
+                        const float gv = __ldg(A.ghost + (int64_t)g * A.nslots + slot);
+                        if (A.mesh.bc[g] == 2) {
+                            const float *rw = A.rhow + ((int64_t)g * A.nfmax + face_elem(A.mesh, ec, d)) * NQ + N1 * w;
+#pragma unroll
+                            for (int ln = 0; ln < N1; ln++)
+                                tF[ln] = gv * __ldg(rw + ln);
+                        } else {
+#pragma unroll
+                            for (int ln = 0; ln < N1; ln++)
+                                tF[ln] = gv;
+                        }
+                    }
+                }
+                float gS[N1];  // the staged side's ghost value of every line on a boundary face
+#pragma unroll
+                for (int ln = 0; ln < N1; ln++)
+                    gS[ln] = 0.f;
+                if (GEN && es < 0) {
+                    const int g = 2 * d + (lo ? 0 : 1);
                     const float gv = __ldg(A.ghost + (int64_t)g * A.nslots + slot);
                     if (A.mesh.bc[g] == 2) {
                         const float *rw = A.rhow + ((int64_t)g * A.nfmax + face_elem(A.mesh, ec, d)) * NQ + N1 * w;
 #pragma unroll
                         for (int ln = 0; ln < N1; ln++)
-                            tF[ln] = gv * __ldg(rw + ln);
+                            gS[ln] = gv * __ldg(rw + ln);
                     } else {
 #pragma unroll
                         for (int ln = 0; ln < N1; ln++)
-                            tF[ln] = gv;
+                            gS[ln] = gv;
                     }
                 }
-            }
-            float gS[N1];  // the staged side's ghost value of every line on a boundary face
+                if constexpr (N1 % 2 == 0) {
+                    // two adjacent lines at a time on packed FP32 pairs: the same operations, in the same
+                    // order, as curv_line_c on each line (bit-identical results)
+                    const unsigned long long X0 = pack2(x0, x0), X1 = pack2(x1, x1), X2 = pack2(x2, x2);
 #pragma unroll
-            for (int ln = 0; ln < N1; ln++)
-                gS[ln] = 0.f;
-            if (GEN && es < 0) {
-                const int g = 2 * d + (lo ? 0 : 1);
-                const float gv = __ldg(A.ghost + (int64_t)g * A.nslots + slot);
-                if (A.mesh.bc[g] == 2) {
-                    const float *rw = A.rhow + ((int64_t)g * A.nfmax + face_elem(A.mesh, ec, d)) * NQ + N1 * w;
+                    for (int ln = 0; ln < N1; ln += 2) {
+                        unsigned long long fl[N1], F[N1], v[N1], sp[N1];
 #pragma unroll
-                    for (int ln = 0; ln < N1; ln++)
-                        gS[ln] = gv * __ldg(rw + ln);
+                        for (int j = 0; j < N1; j++) {
+                            fl[j] = pack2(sm.fs[b][node(ln, j)][lane], sm.fs[b][node(ln + 1, j)][lane]);
+                            v[j] = pack2(sm.sl[w][ks][srow(ln, j)][lane], sm.sl[w][ks][srow(ln + 1, j)][lane]);
+                            const float4 *mp = &sm.metp[d][pair_row<N1>(d, node(ln, j))][0];
+                            const float4 p0 = mp[0], p1 = mp[1];
+                            const unsigned long long u =
+                                ffma2(pack2(p1.x, p1.y), X2, ffma2(pack2(p0.z, p0.w), X1, fmul2(pack2(p0.x, p0.y), X0)));
+                            F[j] = fmul2(u, fl[j]);
+                            sp[j] = pack2(p1.z, p1.w);
+                        }
+                        // the staged side's trace of both lines, and their own traces
+                        unsigned long long t = 0ull, oL = 0ull, oR = 0ull;
+#pragma unroll
+                        for (int j = 1; j < N1; j++)
+                            t = ffma2(dup2(cS[j]), fsub2(v[j], v[0]), t);
+                        t = fadd2(v[0], t);
+#pragma unroll
+                        for (int j = 0; j < N1; j++) {
+                            oL = ffma2(dup2(A.ops.lm[j]), fl[j], oL);
+                            oR = ffma2(dup2(A.ops.lp[j]), fl[j], oR);
+                        }
+                        float tS2[2], oL2[2], oR2[2], FI[2][2];
+                        unpack2(t, tS2[0], tS2[1]);
+                        unpack2(oL, oL2[0], oL2[1]);
+                        unpack2(oR, oR2[0], oR2[1]);
+#pragma unroll
+                        for (int h = 0; h < 2; h++) {
+                            const float tS = !GEN || es >= 0 ? tS2[h] : gS[ln + h];
+                            const float tL = lo ? tS : tF[ln + h], tR = lo ? tF[ln + h] : tS;
+                            FI[0][h] = uL[ln + h] * (uL[ln + h] > 0.f ? tL : oL2[h]);
+                            FI[1][h] = uR[ln + h] * (uR[ln + h] < 0.f ? tR : oR2[h]);
+                        }
+                        const unsigned long long FIL = pack2(FI[0][0], FI[0][1]), FIR = pack2(FI[1][0], FI[1][1]);
+#pragma unroll
+                        for (int i = 0; i < N1; i++) {
+                            unsigned long long a = ffma2(dup2(A.ops.gl[i]), FIL, fmul2(dup2(A.ops.gr[i]), FIR));
+#pragma unroll
+                            for (int j = 0; j < N1; j++)
+                                a = ffma2(dup2(A.ops.DM[i][j]), F[j], a);
+                            float sa, sb;
+                            unpack2(a, sa, sb);
+                            if (d < 2) {
+                                float ca, cb;
+                                unpack2(sp[i], ca, cb);
+                                acc[node(ln, i) - NQ * w] = fmaf(ca, sa, acc[node(ln, i) - NQ * w]);
+                                acc[node(ln + 1, i) - NQ * w] = fmaf(cb, sb, acc[node(ln + 1, i) - NQ * w]);
+                            } else {
+                                sm.fs[b][node(ln, i)][lane] = sa;
+                                sm.fs[b][node(ln + 1, i)][lane] = sb;
+                            }
+                        }
+                    }
                 } else {
 #pragma unroll
-                    for (int ln = 0; ln < N1; ln++)
-                        gS[ln] = gv;
-                }
-            }
-            if constexpr (N1 % 2 == 0) {
-                // two adjacent lines at a time on packed FP32 pairs: the same operations, in the same
-                // order, as curv_line_c on each line (bit-identical results)
-                const unsigned long long X0 = pack2(x0, x0), X1 = pack2(x1, x1), X2 = pack2(x2, x2);
+                    for (int ln = 0; ln < N1; ln++) {
+                        float fl[N1], u[N1], sv[N1], v[N1];
 #pragma unroll
-                for (int ln = 0; ln < N1; ln += 2) {
-                    unsigned long long fl[N1], F[N1], v[N1], sp[N1];
+                        for (int j = 0; j < N1; j++) {
+                            fl[j] = sm.fs[b][node(ln, j)][lane];
+                            v[j] = sm.sl[w][ks][srow(ln, j)][lane];
+                            const float4 m = sm.met[node(ln, j)][d];
+                            u[j] = fmaf(m.z, x2, fmaf(m.y, x1, m.x * x0));
+                        }
+                        const float tS = !GEN || es >= 0 ? trace(v, cS) : gS[ln];
+                        curv_line_c<N1>(sv, fl, u, uL[ln], uR[ln], lo ? tS : tF[ln], lo ? tF[ln] : tS, A.ops);
 #pragma unroll
-                    for (int j = 0; j < N1; j++) {
-                        fl[j] = pack2(sm.fs[b][node(ln, j)][lane], sm.fs[b][node(ln + 1, j)][lane]);
-                        v[j] = pack2(sm.sl[w][ks][srow(ln, j)][lane], sm.sl[w][ks][srow(ln + 1, j)][lane]);
-                        const float4 *mp = &sm.metp[d][pair_row<N1>(d, node(ln, j))][0];
-                        const float4 p0 = mp[0], p1 = mp[1];
-                        const unsigned long long u =
-                            ffma2(pack2(p1.x, p1.y), X2, ffma2(pack2(p0.z, p0.w), X1, fmul2(pack2(p0.x, p0.y), X0)));
-                        F[j] = fmul2(u, fl[j]);
-                        sp[j] = pack2(p1.z, p1.w);
-                    }
-                    // the staged side's trace of both lines, and their own traces
-                    unsigned long long t = 0ull, oL = 0ull, oR = 0ull;
-#pragma unroll
-                    for (int j = 1; j < N1; j++)
-                        t = ffma2(dup2(cS[j]), fsub2(v[j], v[0]), t);
-                    t = fadd2(v[0], t);
-#pragma unroll
-                    for (int j = 0; j < N1; j++) {
-                        oL = ffma2(dup2(A.ops.lm[j]), fl[j], oL);
-                        oR = ffma2(dup2(A.ops.lp[j]), fl[j], oR);
-                    }
-                    float tS2[2], oL2[2], oR2[2], FI[2][2];
-                    unpack2(t, tS2[0], tS2[1]);
-                    unpack2(oL, oL2[0], oL2[1]);
-                    unpack2(oR, oR2[0], oR2[1]);
-#pragma unroll
-                    for (int h = 0; h < 2; h++) {
-                        const float tS = !GEN || es >= 0 ? tS2[h] : gS[ln + h];
-                        const float tL = lo ? tS : tF[ln + h], tR = lo ? tF[ln + h] : tS;
-                        FI[0][h] = uL[ln + h] * (uL[ln + h] > 0.f ? tL : oL2[h]);
-                        FI[1][h] = uR[ln + h] * (uR[ln + h] < 0.f ? tR : oR2[h]);
-                    }
-                    const unsigned long long FIL = pack2(FI[0][0], FI[0][1]), FIR = pack2(FI[1][0], FI[1][1]);
-#pragma unroll
-                    for (int i = 0; i < N1; i++) {
-                        unsigned long long a = ffma2(dup2(A.ops.gl[i]), FIL, fmul2(dup2(A.ops.gr[i]), FIR));
-#pragma unroll
-                        for (int j = 0; j < N1; j++)
-                            a = ffma2(dup2(A.ops.DM[i][j]), F[j], a);
-                        float sa, sb;
-                        unpack2(a, sa, sb);
-                        if (d < 2) {
-                            float ca, cb;
-                            unpack2(sp[i], ca, cb);
-                            acc[node(ln, i) - NQ * w] = fmaf(ca, sa, acc[node(ln, i) - NQ * w]);
-                            acc[node(ln + 1, i) - NQ * w] = fmaf(cb, sb, acc[node(ln + 1, i) - NQ * w]);
-                        } else {
-                            sm.fs[b][node(ln, i)][lane] = sa;
-                            sm.fs[b][node(ln + 1, i)][lane] = sb;
+                        for (int j = 0; j < N1; j++) {
+                            if (d < 2)
+                                acc[node(ln, j) - NQ * w] = fmaf(sm.met[node(ln, j)][0].w, sv[j], acc[node(ln, j) - NQ * w]);
+                            else
+                                sm.fs[b][node(ln, j)][lane] = sv[j];
                         }
                     }
                 }
-            } else {
-#pragma unroll
-                for (int ln = 0; ln < N1; ln++) {
-                    float fl[N1], u[N1], sv[N1], v[N1];
-#pragma unroll
-                    for (int j = 0; j < N1; j++) {
-                        fl[j] = sm.fs[b][node(ln, j)][lane];
-                        v[j] = sm.sl[w][ks][srow(ln, j)][lane];
-                        const float4 m = sm.met[node(ln, j)][d];
-                        u[j] = fmaf(m.z, x2, fmaf(m.y, x1, m.x * x0));
-                    }
-                    const float tS = !GEN || es >= 0 ? trace(v, cS) : gS[ln];
-                    curv_line_c<N1>(sv, fl, u, uL[ln], uR[ln], lo ? tS : tF[ln], lo ? tF[ln] : tS, A.ops);
-#pragma unroll
-                    for (int j = 0; j < N1; j++) {
-                        if (d < 2)
-                            acc[node(ln, j) - NQ * w] = fmaf(sm.met[node(ln, j)][0].w, sv[j], acc[node(ln, j) - NQ * w]);
-                        else
-                            sm.fs[b][node(ln, j)][lane] = sv[j];
-                    }
+            };
+            wait(2 + kx);
+            lines(std::integral_constant<int, 0>{}, kx, l0, enx);
+            wait(2 + ky);
+            lines(std::integral_constant<int, 1>{}, ky, l1, eny);
+            // slots kx and ky are consumed: the next tile's f^n and x-neighbour layer land there
+            __syncwarp();
+            if (more && ((lane == RFN && has_fn) || lane == RX)) {
+                fence_proxy_async();
+                issue_layer(lane == RX && turn ? role_src(enn) : csrc, vl + 1, lane == RX ? ky : kx);
+            }
+            __syncthreads();  // B1: every layer of the element tile has landed
+            // z-lines of slice iy = w (all layers) from the shared tile
+            wait(2 + ka);
+            lines(std::integral_constant<int, 2>{}, ka, l2, enz);
+            // slot ka is consumed: the next tile's y-neighbour layer lands there; warp 0 also brings the next
+            // tile's velocity table into the other table buffer (every warp is past B1)
+            __syncwarp();
+            if (more && (lane == RY || (w == 0 && lane == RT))) {
+                fence_proxy_async();
+                if (lane == RY) {
+                    issue_layer(turn ? role_src(enn) : csrc, vl + 1, ka);
+                } else {
+                    mbar_arrive_expect_tx(tbar(b ^ 1), kTabRows * kRow);
+                    bulk_g2s(smem_u32(&sm.tab[b ^ 1][0][0]), A.vtab + (int64_t)(vt + 1) * kTabRows * kWarp,
+                             kTabRows * kRow, tbar(b ^ 1));
                 }
             }
-        };
-        wait(2 + kx);
-        lines(std::integral_constant<int, 0>{}, kx, l0, enx);
-        wait(2 + ky);
-        lines(std::integral_constant<int, 1>{}, ky, l1, eny);
-        // slots kx and ky are consumed: the next tile's f^n and x-neighbour layer land there
-        __syncwarp();
-        if (more && ((lane == RFN && has_fn) || lane == RX)) {
-            fence_proxy_async();
-            issue_layer(lane == RX && turn ? role_src(enn) : csrc, vl + 1, lane == RX ? ky : kx);
-        }
-        __syncthreads();  // B1: every layer of the element tile has landed
-        // z-lines of slice iy = w (all layers) from the shared tile
-        wait(2 + ka);
-        lines(std::integral_constant<int, 2>{}, ka, l2, enz);
-        // slot ka is consumed: the next tile's y-neighbour layer lands there; warp 0 also brings the next
-        // tile's velocity table into the other table buffer (every warp is past B1)
-        __syncwarp();
-        if (more && (lane == RY || (w == 0 && lane == RT))) {
-            fence_proxy_async();
-            if (lane == RY) {
-                issue_layer(turn ? role_src(enn) : csrc, vl + 1, ka);
-            } else {
-                mbar_arrive_expect_tx(tbar(b ^ 1), kTabRows * kRow);
-                bulk_g2s(smem_u32(&sm.tab[b ^ 1][0][0]), A.vtab + (int64_t)(vt + 1) * kTabRows * kWarp,
-                         kTabRows * kRow, tbar(b ^ 1));
-            }
-        }
-        __syncthreads();  // B2: z-sums complete
-#pragma unroll
-        for (int q = 0; q < NQ; q++)
-            acc[q] = fmaf(sm.met[q + NQ * w][0].w, sm.fs[b][q + NQ * w][lane], acc[q]);
-        __syncwarp();  // the z-sums of this layer are read before its rows take the stage output
-        const float gm = sm.tab[b][3][lane] != 0.f ? 1.f : 0.f;
-        const float cg = A.kg * gm, cf = bdt * gm;
-        const float xs = x0 * x0 + x1 * x1 + x2 * x2;
-        const float mm0 = m0 * m0, mm1 = m1 * m1, mm2 = m2 * m2, mms = mm0 + mm1 + mm2;
-        const bool iso = !GEN || A.viso;
-        const unsigned long long M0 = pack2(m0, m0), M1 = pack2(m1, m1), M2 = pack2(m2, m2);
-        const unsigned long long U0 = iso ? pack2(mms, mms) : pack2(mm0, mm0);
-        const unsigned long long U1 = iso ? U0 : pack2(mm1, mm1);
-        const unsigned long long U2 = iso ? 0ull : pack2(mm2, mm2);
-        float *dst = A.dst + fidx(vl, e, 0, lane, E, NP);
-        float lsum = 0.f, lmin = 3.4e38f;
-        auto bgk_src = [&](auto vtau_c, auto force_c, auto lim_c) {
-            constexpr bool VT = decltype(vtau_c)::value, FP = decltype(force_c)::value;
-            constexpr bool LIM = decltype(lim_c)::value;
-#pragma unroll
-            for (int h = 0; h < (NQ + 1) / 2; h++) {
-                const float4 *pp = reinterpret_cast<const float4 *>(&sm.par[w][h][0][0]);
-                const float4 p01 = pp[0], p23 = pp[1], p45 = pp[2], p67 = pp[3];
-                const unsigned long long lin =
-                    ffma2(pack2(p23.z, p23.w), M2,
-                          ffma2(pack2(p23.x, p23.y), M1, ffma2(pack2(p01.z, p01.w), M0, pack2(p01.x, p01.y))));
-                const unsigned long long ex =
-                    GEN ? ffma2(pack2(p45.x, p45.y), U0,
-                                ffma2(pack2(p45.z, p45.w), U1, ffma2(pack2(p67.x, p67.y), U2, lin)))
-                        : ffma2(pack2(p45.x, p45.y), U0, ffma2(pack2(p45.z, p45.w), U0, lin));
-                float g[2];
-                exp2_fp32x2(ex, pack2(p67.z, p67.w), g[0], g[1]);
-#pragma unroll
-                for (int sl = 0; sl < 2; sl++) {
-                    const int q = 2 * h + sl;
-                    if (q >= NQ)
-                        break;
-                    const int i = q + NQ * w;
-                    const float a = acc[q];
-                    float gc = cg;
-                    if constexpr (VT) {
-                        const float itau = sl == 0 ? p67.x : p67.y;
-                        gc = __fsub_rn(A.b, __fsub_rn(A.b, __fmul_rn(bdt, itau))) * gm;
-                    }
-                    if constexpr (FP) {
-                        const float4 fq = *reinterpret_cast<const float4 *>(&sm.fpar[i][0]);
-                        const float qv =
-                            fmaf(sm.fpar[i][4], xs, fmaf(fq.w, x2, fmaf(fq.z, x1, fmaf(fq.y, x0, fq.x))));
-                        gc = fmaf(cf, qv, gc);  // on top of the node's own Maxwellian weight
-                    }
-                    const float o = fmaf(gc, g[sl], a);
-                    if constexpr (LIM) {
-                        lsum = fmaf(sm.met[i][1].w, o, lsum);
-                        lmin = fminf(lmin, o);
-                    } else {
-                        __stcs(dst + i * kWarp, o);
-                    }
-                    sm.fs[b][q + NQ * w][lane ^ (4 * (q & 7))] = o;
-                }
-            }
-        };
-        using T_ = std::true_type;
-        using F_ = std::false_type;
-        if constexpr (GEN) {
-            if (A.limiter) {
-                if (A.fpar)
-                    A.vtau ? bgk_src(T_{}, T_{}, T_{}) : bgk_src(F_{}, T_{}, T_{});
-                else
-                    A.vtau ? bgk_src(T_{}, F_{}, T_{}) : bgk_src(F_{}, F_{}, T_{});
-            } else {
-                if (A.fpar)
-                    A.vtau ? bgk_src(T_{}, T_{}, F_{}) : bgk_src(F_{}, T_{}, F_{});
-                else
-                    A.vtau ? bgk_src(T_{}, F_{}, F_{}) : bgk_src(F_{}, F_{}, F_{});
-            }
-        } else {
-            bgk_src(F_{}, F_{}, F_{});
-        }
-        if (GEN && A.limiter) {
-            // Zhang-Shu (Sec. 2.1, Eqs. 10-11) over the physical element: weights W J over their sum
-            sm.lim[0][w][lane] = lsum;
-            sm.lim[1][w][lane] = lmin;
-            __syncthreads();  // B3
-            float mean = 0.f, mn = sm.lim[1][0][lane];
-#pragma unroll
-            for (int lw = 0; lw < N1; lw++) {
-                mean += sm.lim[0][lw][lane];
-                mn = fminf(mn, sm.lim[1][lw][lane]);
-            }
-            mean *= sm.iwj;
-            const float beta = mn < 0.f ? fminf(fabsf(mean / (mean - mn)), 1.f) : 1.f;
-            if (mn < 0.f) {
-#pragma unroll
-                for (int q = 0; q < NQ; q++) {
-                    float &slot_o = sm.fs[b][q + NQ * w][lane ^ (4 * (q & 7))];
-                    slot_o = fmaf(beta, slot_o - mean, mean);
-                }
-            }
+            __syncthreads();  // B2: z-sums complete
 #pragma unroll
             for (int q = 0; q < NQ; q++)
-                __stcs(dst + (q + NQ * w) * kWarp, sm.fs[b][q + NQ * w][lane ^ (4 * (q & 7))]);
-        }
-        // moments of this layer's nodes (Eq. 2 with Eq. 12) of the stored values
-        __syncwarp();
-        unsigned long long pm[2][5];
+                acc[q] = fmaf(sm.met[q + NQ * w][0].w, sm.fs[b][q + NQ * w][lane], acc[q]);
+            __syncwarp();  // the z-sums of this layer are read before its rows take the stage output
+            const float gm = sm.tab[b][3][lane] != 0.f ? 1.f : 0.f;
+            const float cg = A.kg * gm, cf = bdt * gm;
+            const float xs = x0 * x0 + x1 * x1 + x2 * x2;
+            const float mm0 = m0 * m0, mm1 = m1 * m1, mm2 = m2 * m2, mms = mm0 + mm1 + mm2;
+            const bool iso = !GEN || A.viso;
+            const unsigned long long M0 = pack2(m0, m0), M1 = pack2(m1, m1), M2 = pack2(m2, m2);
+            const unsigned long long U0 = iso ? pack2(mms, mms) : pack2(mm0, mm0);
+            const unsigned long long U1 = iso ? U0 : pack2(mm1, mm1);
+            const unsigned long long U2 = iso ? 0ull : pack2(mm2, mm2);
+            float *dst = A.dst + fidx(vl, e, 0, lane, E, NP);
+            float lsum = 0.f, lmin = 3.4e38f;
+            auto bgk_src = [&](auto vtau_c, auto force_c, auto lim_c) {
+                constexpr bool VT = decltype(vtau_c)::value, FP = decltype(force_c)::value;
+                constexpr bool LIM = decltype(lim_c)::value;
 #pragma unroll
-        for (int h = 0; h < NHR; h++)
+                for (int h = 0; h < (NQ + 1) / 2; h++) {
+                    const float4 *pp = reinterpret_cast<const float4 *>(&sm.par[w][h][0][0]);
+                    const float4 p01 = pp[0], p23 = pp[1], p45 = pp[2], p67 = pp[3];
+                    const unsigned long long lin =
+                        ffma2(pack2(p23.z, p23.w), M2,
+                              ffma2(pack2(p23.x, p23.y), M1, ffma2(pack2(p01.z, p01.w), M0, pack2(p01.x, p01.y))));
+                    const unsigned long long ex =
+                        GEN ? ffma2(pack2(p45.x, p45.y), U0,
+                                    ffma2(pack2(p45.z, p45.w), U1, ffma2(pack2(p67.x, p67.y), U2, lin)))
+                            : ffma2(pack2(p45.x, p45.y), U0, ffma2(pack2(p45.z, p45.w), U0, lin));
+                    float g[2];
+                    exp2_fp32x2(ex, pack2(p67.z, p67.w), g[0], g[1]);
 #pragma unroll
-            for (int c = 0; c < 5; c++)
-                pm[h][c] = 0ull;
+                    for (int sl = 0; sl < 2; sl++) {
+                        const int q = 2 * h + sl;
+                        if (q >= NQ)
+                            break;
+                        const int i = q + NQ * w;
+                        const float a = acc[q];
+                        float gc = cg;
+                        if constexpr (VT) {
+                            const float itau = sl == 0 ? p67.x : p67.y;
+                            gc = __fsub_rn(A.b, __fsub_rn(A.b, __fmul_rn(bdt, itau))) * gm;
+                        }
+                        if constexpr (FP) {
+                            const float4 fq = *reinterpret_cast<const float4 *>(&sm.fpar[i][0]);
+                            const float qv =
+                                fmaf(sm.fpar[i][4], xs, fmaf(fq.w, x2, fmaf(fq.z, x1, fmaf(fq.y, x0, fq.x))));
+                            gc = fmaf(cf, qv, gc);  // on top of the node's own Maxwellian weight
+                        }
+                        const float o = fmaf(gc, g[sl], a);
+                        if constexpr (LIM) {
+                            lsum = fmaf(sm.met[i][1].w, o, lsum);
+                            lmin = fminf(lmin, o);
+                        } else {
+                            __stcs(dst + i * kWarp, o);
+                        }
+                        sm.fs[b][q + NQ * w][lane ^ (4 * (q & 7))] = o;
+                    }
+                }
+            };
+            using T_ = std::true_type;
+            using F_ = std::false_type;
+            if constexpr (GEN) {
+                if (A.limiter) {
+                    if (A.fpar)
+                        A.vtau ? bgk_src(T_{}, T_{}, T_{}) : bgk_src(F_{}, T_{}, T_{});
+                    else
+                        A.vtau ? bgk_src(T_{}, F_{}, T_{}) : bgk_src(F_{}, F_{}, T_{});
+                } else {
+                    if (A.fpar)
+                        A.vtau ? bgk_src(T_{}, T_{}, F_{}) : bgk_src(F_{}, T_{}, F_{});
+                    else
+                        A.vtau ? bgk_src(T_{}, F_{}, F_{}) : bgk_src(F_{}, F_{}, F_{});
+                }
+            } else {
+                bgk_src(F_{}, F_{}, F_{});
+            }
+            if (GEN && A.limiter) {
+                // Zhang-Shu (Sec. 2.1, Eqs. 10-11) over the physical element: weights W J over their sum
+                sm.lim[0][w][lane] = lsum;
+                sm.lim[1][w][lane] = lmin;
+                __syncthreads();  // B3
+                float mean = 0.f, mn = sm.lim[1][0][lane];
 #pragma unroll
-        for (int k = 0; k < 8; k += 4) {
-            const int kk = 8 * kg + k;
-            unsigned long long wv[5][2];
-            {
-                const float4 W4 = *reinterpret_cast<const float4 *>(&sm.tab[b][3][kk]);
-                const float4 E4 = *reinterpret_cast<const float4 *>(&sm.tab[b][4][kk]);
-                wv[0][0] = pack2(W4.x, W4.y);
-                wv[0][1] = pack2(W4.z, W4.w);
-                wv[4][0] = pack2(E4.x, E4.y);
-                wv[4][1] = pack2(E4.z, E4.w);
+                for (int lw = 0; lw < N1; lw++) {
+                    mean += sm.lim[0][lw][lane];
+                    mn = fminf(mn, sm.lim[1][lw][lane]);
+                }
+                mean *= sm.iwj;
+                const float beta = mn < 0.f ? fminf(fabsf(mean / (mean - mn)), 1.f) : 1.f;
+                if (mn < 0.f) {
 #pragma unroll
-                for (int d = 0; d < 3; d++) {
-                    const float4 M4 = *reinterpret_cast<const float4 *>(&sm.tab[b][d][kk]);
-                    wv[1 + d][0] = fmul2(pack2(W4.x, W4.y), pack2(M4.x, M4.y));
-                    wv[1 + d][1] = fmul2(pack2(W4.z, W4.w), pack2(M4.z, M4.w));
+                    for (int q = 0; q < NQ; q++) {
+                        float &slot_o = sm.fs[b][q + NQ * w][lane ^ (4 * (q & 7))];
+                        slot_o = fmaf(beta, slot_o - mean, mean);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < NQ; q++)
+                    __stcs(dst + (q + NQ * w) * kWarp, sm.fs[b][q + NQ * w][lane ^ (4 * (q & 7))]);
+            }
+            // moments of this layer's nodes (Eq. 2 with Eq. 12) of the stored values
+            __syncwarp();
+            unsigned long long pm[2][5];
+#pragma unroll
+            for (int h = 0; h < NHR; h++)
+#pragma unroll
+                for (int c = 0; c < 5; c++)
+                    pm[h][c] = 0ull;
+#pragma unroll
+            for (int k = 0; k < 8; k += 4) {
+                const int kk = 8 * kg + k;
+                unsigned long long wv[5][2];
+                {
+                    const float4 W4 = *reinterpret_cast<const float4 *>(&sm.tab[b][3][kk]);
+                    const float4 E4 = *reinterpret_cast<const float4 *>(&sm.tab[b][4][kk]);
+                    wv[0][0] = pack2(W4.x, W4.y);
+                    wv[0][1] = pack2(W4.z, W4.w);
+                    wv[4][0] = pack2(E4.x, E4.y);
+                    wv[4][1] = pack2(E4.z, E4.w);
+#pragma unroll
+                    for (int d = 0; d < 3; d++) {
+                        const float4 M4 = *reinterpret_cast<const float4 *>(&sm.tab[b][d][kk]);
+                        wv[1 + d][0] = fmul2(pack2(W4.x, W4.y), pack2(M4.x, M4.y));
+                        wv[1 + d][1] = fmul2(pack2(W4.z, W4.w), pack2(M4.z, M4.w));
+                    }
+                }
+#pragma unroll
+                for (int h = 0; h < NHR; h++) {
+                    const int row = min(np + 8 * h, NQ - 1);
+                    const float4 v = *reinterpret_cast<const float4 *>(&sm.fs[b][row + NQ * w][kk ^ (4 * (row & 7))]);
+                    const unsigned long long v01 = pack2(v.x, v.y), v23 = pack2(v.z, v.w);
+#pragma unroll
+                    for (int c = 0; c < 5; c++) {
+                        pm[h][c] = ffma2(wv[c][0], v01, pm[h][c]);
+                        pm[h][c] = ffma2(wv[c][1], v23, pm[h][c]);
+                    }
                 }
             }
 #pragma unroll
-            for (int h = 0; h < NHR; h++) {
-                const int row = min(np + 8 * h, NQ - 1);
-                const float4 v = *reinterpret_cast<const float4 *>(&sm.fs[b][row + NQ * w][kk ^ (4 * (row & 7))]);
-                const unsigned long long v01 = pack2(v.x, v.y), v23 = pack2(v.z, v.w);
+            for (int h = 0; h < NHR; h++)
 #pragma unroll
-                for (int c = 0; c < 5; c++) {
-                    pm[h][c] = ffma2(wv[c][0], v01, pm[h][c]);
-                    pm[h][c] = ffma2(wv[c][1], v23, pm[h][c]);
-                }
+                for (int c = 0; c < 5; c++)
+                    msum[h][c] += sum2(pm[h][c]);
+#pragma unroll
+            for (int d = 0; d < 3; d++)
+                en[d] = enn[d];
+            if (turn) {
+                csrc = role_src(en);
+                octc = octn;
             }
+            ka = ka == 2 ? 0 : ka + 1;
         }
-#pragma unroll
-        for (int h = 0; h < NHR; h++)
-#pragma unroll
-            for (int c = 0; c < 5; c++)
-                msum[h][c] += sum2(pm[h][c]);
-#pragma unroll
-        for (int d = 0; d < 3; d++)
-            en[d] = enn[d];
-        if (turn) {
-            csrc = role_src(en);
-            octc = octn;
-        }
-        ka = ka == 2 ? 0 : ka + 1;
-        if (vl + 1 == ge) {
-            const int grp = moment_group(A, blockIdx.x / E, vl);
+            const int grp = moment_group(A, blockIdx.x / E, vl - 1);
 #pragma unroll
             for (int h = 0; h < NHR; h++) {
                 const int q = np + 8 * h;
@@ -697,7 +698,6 @@ __global__ void __launch_bounds__(kWarp *N1, (N1 >= 4 ? BGK_STAGE3C_MINCTAS_P3 :
                 }
             }
             ge = min(ge + A.G, vl1);
-        }
     }
 }
 
