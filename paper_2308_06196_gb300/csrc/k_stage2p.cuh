@@ -139,275 +139,276 @@ __global__ void __launch_bounds__(kWarp *kStage2pWarps<N1>, kStage2pResident<N1>
     auto ld2 = [](const float *p) { return *reinterpret_cast<const u64 *>(p); };
     auto st2 = [](float *p, u64 v) { *reinterpret_cast<u64 *>(p) = v; };
 
-    for (int vl = vl0; vl < vl1; vl++) {
-        const int vt = A.vt0 + vl;
-        const int b = (vl - vl0) & 1;
-        const bool more = vl + 1 < vl1;
-        const int oct = octc, octn = OCT < 8 ? OCT : (more ? (int)__ldg(A.toct + vt + 1) : octc);
-        const bool turn = OCT == 8 && octn != oct;
-        const float *nsrc = csrc;  // this role lane's source of the next tile
-        if (turn && role)
-            nsrc = role_src(octn);
-        float(*const F)[kWarp] = sm.buf[bF];
-        const float(*const pN)[kWarp] = sm.buf[bN] + row0, (*const pX)[kWarp] = sm.buf[bX] + row0,
-                         (*const pY)[kWarp] = sm.buf[bY] + row0;
-        wait(bF);
-        mbar_wait(tbar(b), (ph >> (4 + b)) & 1, A.err);
-        ph ^= 1u << (4 + b);
-        float m[3][2], x[2][2];
-        u64 cdir[2];
-#pragma unroll
-        for (int d = 0; d < 3; d++)
-            unpack2(ld2(&sm.tab[b][d][c2]), m[d][0], m[d][1]);
-#pragma unroll
-        for (int d = 0; d < 2; d++) {
-#pragma unroll
-            for (int s = 0; s < 2; s++)
-                x[d][s] = fmaf(A.vs[d], m[d][s], A.vc[d]);
-            cdir[d] = pack2(-A.mesh.inv_h2[d] * x[d][0] * bdt, -A.mesh.inv_h2[d] * x[d][1] * bdt);
-        }
-        u64 f[NQ], acc[NQ];
-#pragma unroll
-        for (int q = 0; q < NQ; q++)
-            f[q] = ld2(&F[row0 + q][c2]);
-        // acc = an f^n + b (1 - dt/tau) f_s
-        if (GEN && A.vtau) {
-#pragma unroll
-            for (int q = 0; q < NQ; q++)
-                acc[q] = fmul2(dup2(__fsub_rn(A.b, __fmul_rn(bdt, sm.par[hf * Sm::kParElem + q * kParamStride + 6]))), f[q]);
-        } else {
-            const u64 kb = dup2(A.kb);
-#pragma unroll
-            for (int q = 0; q < NQ; q++)
-                acc[q] = fmul2(kb, f[q]);
-        }
-        if (has_fn) {
-            wait(bN);
-            const u64 an = dup2(A.an);
-#pragma unroll
-            for (int q = 0; q < NQ; q++)
-                acc[q] = ffma2(an, ld2(&pN[q][c2]), acc[q]);
-        }
-        __syncwarp();  // f^n is consumed: the next tile's x-neighbour; the other table buffer: its table
-        if (more && ((role && op == 2) || lane == 8)) {
-            fence_proxy_async();
-            if (lane == 8)
-                issue_table(vl + 1, b ^ 1);
-            else
-                issue(nsrc, vl + 1, bN);
-        }
-        // The lines of one direction: line k's nodes f[line(k, j)], its upwind neighbour's row nb(k, j); where
-        // that is no element (a Dirichlet ghost) the jump is the ghost's
-        auto lines = [&](auto dc, int en, const float(*nbr)[kWarp], auto row) {
-            constexpr int d = decltype(dc)::value;
-            const bool left = (oct >> d) & 1, inner = GEN == 0 || en >= 0;
-            u64 gh = 0;
-            if (GEN && !inner)
-                gh = *reinterpret_cast<const u64 *>(A.ghost + (2 * d + (left ? 0 : 1)) * A.nslots + vt * kWarp + c2);
-#pragma unroll
-            for (int k = 0; k < N1; k++) {
-                u64 fl[N1], sv[N1], v[N1];
-#pragma unroll
-                for (int j = 0; j < N1; j++) {
-                    fl[j] = f[row(k, j)];
-                    v[j] = ld2(&nbr[row(k, j)][c2]);
-                }
-                auto side = [&](auto left_c) {
-                    constexpr bool LEFT = decltype(left_c)::value;
-                    constexpr int R = LEFT ? 0 : N1 - 1;
-                    const u64 tj = trace_jump2<N1, LEFT>(v, fl[R], A.ops);
-                    const u64 tr = GEN == 0 ? tj : (inner ? tj : fsub2(gh, fl[R]));  // (per element: a select)
-                    line_sums_jump2<N1, LEFT>(sv, fl, tr, A.ops);
-                };
-                if (left)
-                    side(std::true_type{});
-                else
-                    side(std::false_type{});
-#pragma unroll
-                for (int j = 0; j < N1; j++)
-                    acc[row(k, j)] = ffma2(cdir[d], sv[j], acc[row(k, j)]);
-            }
-        };
-        wait(bX);
-        lines(std::integral_constant<int, 0>{}, enx, pX, [](int k, int j) { return j + N1 * k; });
-        __syncwarp();  // the x-neighbour is consumed: the next tile's f_s
-        if (more && role && op == 0) {
-            fence_proxy_async();
-            issue(csrc, vl + 1, bX);
-        }
-        wait(bY);
-        lines(std::integral_constant<int, 1>{}, eny, pY, [](int k, int j) { return k + N1 * j; });
-        __syncwarp();  // the y-neighbour is consumed: the next tile's f^n
-        if (more && has_fn && role && op == 1) {
-            fence_proxy_async();
-            issue(csrc, vl + 1, bY);
-        }
-        // BGK source towards the conservative Maxwellian, Shu-Osher combination, store
-        float W0, W1;
-        unpack2(ld2(&sm.tab[b][3][c2]), W0, W1);
-        const float gm[2] = {W0 != 0.f ? 1.f : 0.f, W1 != 0.f ? 1.f : 0.f};  // the padding mask
-        const bool iso = !GEN || A.viso;
-        float mm[3][2], mms[2];
-#pragma unroll
-        for (int s = 0; s < 2; s++) {
+    for (int vl = vl0; vl < vl1;) {  // a moment group
+        for (; vl < ge; vl++) {
+            const int vt = A.vt0 + vl;
+            const int b = (vl - vl0) & 1;
+            const bool more = vl + 1 < vl1;
+            const int oct = octc, octn = OCT < 8 ? OCT : (more ? (int)__ldg(A.toct + vt + 1) : octc);
+            const bool turn = OCT == 8 && octn != oct;
+            const float *nsrc = csrc;  // this role lane's source of the next tile
+            if (turn && role)
+                nsrc = role_src(octn);
+            float(*const F)[kWarp] = sm.buf[bF];
+            const float(*const pN)[kWarp] = sm.buf[bN] + row0, (*const pX)[kWarp] = sm.buf[bX] + row0,
+                             (*const pY)[kWarp] = sm.buf[bY] + row0;
+            wait(bF);
+            mbar_wait(tbar(b), (ph >> (4 + b)) & 1, A.err);
+            ph ^= 1u << (4 + b);
+            float m[3][2], x[2][2];
+            u64 cdir[2];
 #pragma unroll
             for (int d = 0; d < 3; d++)
-                mm[d][s] = m[d][s] * m[d][s];
-            mms[s] = mm[0][s] + mm[1][s] + mm[2][s];
-            if (iso) {
-                mm[0][s] = mm[1][s] = mms[s];
-                mm[2][s] = 0.f;
+                unpack2(ld2(&sm.tab[b][d][c2]), m[d][0], m[d][1]);
+#pragma unroll
+            for (int d = 0; d < 2; d++) {
+#pragma unroll
+                for (int s = 0; s < 2; s++)
+                    x[d][s] = fmaf(A.vs[d], m[d][s], A.vc[d]);
+                cdir[d] = pack2(-A.mesh.inv_h2[d] * x[d][0] * bdt, -A.mesh.inv_h2[d] * x[d][1] * bdt);
             }
-        }
-        const u64 cg = pack2(A.kg * gm[0], A.kg * gm[1]), gm2 = pack2(gm[0], gm[1]);
-        float *dst = A.dst + fidx(vl, e, 0, c2, E, NQ);
-        auto put_out = [&](int q, u64 o) {  // the stored value, and its transposed copy for the moments
-            if (real)
-                __stcs(reinterpret_cast<u64 *>(dst + q * kWarp), o);
-            st2(&F[row0 + q][c2 ^ (4 * ((q + (NQ % 8 ? NQ * hf : 0)) & 7))], o);  // (its row mod 8)
-        };
-        __syncwarp();  // every lane has read its rows of F
-        auto bgk_src = [&](auto vtau_c, auto lim_c) {
-            constexpr bool VT = decltype(vtau_c)::value, LIM = decltype(lim_c)::value;
-#pragma unroll
-            for (int q = 0; q < NQ; q++) {
-                const float4 *pp = reinterpret_cast<const float4 *>(&sm.par[hf * Sm::kParElem + q * kParamStride]);
-                const float4 pa = pp[0], pb = pp[1];  // (a, b_x, b_y, b_z), (p4, p5, p6, 2^x constant)
-                float ex[2];
-#pragma unroll
-                for (int s = 0; s < 2; s++) {
-                    const float lin = fmaf(pa.w, m[2][s], fmaf(pa.z, m[1][s], fmaf(pa.y, m[0][s], pa.x)));
-                    ex[s] = GEN ? fmaf(pb.x, mm[0][s], fmaf(pb.y, mm[1][s], fmaf(pb.z, mm[2][s], lin)))
-                                : fmaf(pb.x, mms[s], fmaf(pb.y, mms[s], lin));
-                }
-                float g[2];
-                exp2_fp32x2(pack2(ex[0], ex[1]), dup2(pb.w), g[0], g[1]);
-                u64 gc = cg;
-                if constexpr (VT)  // kg = b - kb exactly, kb as in the accumulator above
-                    gc = fmul2(dup2(__fsub_rn(A.b, __fsub_rn(A.b, __fmul_rn(bdt, pb.z)))), gm2);
-                acc[q] = ffma2(gc, pack2(g[0], g[1]), acc[q]);
-                if constexpr (!LIM)
-                    put_out(q, acc[q]);
-            }
-        };
-        using T_ = std::true_type;
-        using F_ = std::false_type;
-        if constexpr (GEN) {
-            if (A.limiter)
-                A.vtau ? bgk_src(T_{}, T_{}) : bgk_src(F_{}, T_{});
-            else
-                A.vtau ? bgk_src(T_{}, F_{}) : bgk_src(F_{}, F_{});
-        } else {
-            bgk_src(F_{}, F_{});
-        }
-        if (GEN && A.limiter) {
-            // Zhang-Shu (Sec. 2.1, Eqs. 10-11): the element mean (tensor Gauss-Legendre weights / 4, summing to
-            // 1) and minimum of each velocity, all in this lane's registers
-            u64 mean2 = 0;
-            float mn[2] = {3.4e38f, 3.4e38f}, mean[2];
-#pragma unroll
-            for (int q = 0; q < NQ; q++) {
-                mean2 = ffma2(dup2(A.ops.wq[q % N1] * A.ops.wq[q / N1]), acc[q], mean2);
-                float o[2];
-                unpack2(acc[q], o[0], o[1]);
-                mn[0] = fminf(mn[0], o[0]);
-                mn[1] = fminf(mn[1], o[1]);
-            }
-            unpack2(mean2, mean[0], mean[1]);
-            float beta[2];
-#pragma unroll
-            for (int s = 0; s < 2; s++)
-                beta[s] = fminf(fabsf(mean[s] / (mean[s] - mn[s])), 1.f);
-            if (mn[0] < 0.f || mn[1] < 0.f) {
-#pragma unroll
-                for (int q = 0; q < NQ; q++) {
-                    float o[2];
-                    unpack2(acc[q], o[0], o[1]);
-#pragma unroll
-                    for (int s = 0; s < 2; s++)
-                        o[s] = mn[s] < 0.f ? fmaf(beta[s], o[s] - mean[s], mean[s]) : o[s];
-                    acc[q] = pack2(o[0], o[1]);
-                }
-            }
+            u64 f[NQ], acc[NQ];
 #pragma unroll
             for (int q = 0; q < NQ; q++)
-                put_out(q, acc[q]);
-        }
-        // moments of the elements' nodes (Eq. 2 with Eq. 12) of the stored values
-        __syncwarp();
-        u64 pm[NR][5];
+                f[q] = ld2(&F[row0 + q][c2]);
+            // acc = an f^n + b (1 - dt/tau) f_s
+            if (GEN && A.vtau) {
 #pragma unroll
-        for (int r = 0; r < NR; r++)
+                for (int q = 0; q < NQ; q++)
+                    acc[q] = fmul2(dup2(__fsub_rn(A.b, __fmul_rn(bdt, sm.par[hf * Sm::kParElem + q * kParamStride + 6]))), f[q]);
+            } else {
+                const u64 kb = dup2(A.kb);
 #pragma unroll
-            for (int c = 0; c < 5; c++)
-                pm[r][c] = 0ull;
+                for (int q = 0; q < NQ; q++)
+                    acc[q] = fmul2(kb, f[q]);
+            }
+            if (has_fn) {
+                wait(bN);
+                const u64 an = dup2(A.an);
 #pragma unroll
-        for (int k = 0; k < 8; k += 4) {
-            const int kk = 8 * kg + k;
-            u64 wv[5][2];
-            {
-                const float4 W4 = *reinterpret_cast<const float4 *>(&sm.tab[b][3][kk]);
-                const float4 E4 = *reinterpret_cast<const float4 *>(&sm.tab[b][4][kk]);
-                wv[0][0] = pack2(W4.x, W4.y);
-                wv[0][1] = pack2(W4.z, W4.w);
-                wv[4][0] = pack2(E4.x, E4.y);
-                wv[4][1] = pack2(E4.z, E4.w);
+                for (int q = 0; q < NQ; q++)
+                    acc[q] = ffma2(an, ld2(&pN[q][c2]), acc[q]);
+            }
+            __syncwarp();  // f^n is consumed: the next tile's x-neighbour; the other table buffer: its table
+            if (more && ((role && op == 2) || lane == 8)) {
+                fence_proxy_async();
+                if (lane == 8)
+                    issue_table(vl + 1, b ^ 1);
+                else
+                    issue(nsrc, vl + 1, bN);
+            }
+            // The lines of one direction: line k's nodes f[line(k, j)], its upwind neighbour's row nb(k, j); where
+            // that is no element (a Dirichlet ghost) the jump is the ghost's
+            auto lines = [&](auto dc, int en, const float(*nbr)[kWarp], auto row) {
+                constexpr int d = decltype(dc)::value;
+                const bool left = (oct >> d) & 1, inner = GEN == 0 || en >= 0;
+                u64 gh = 0;
+                if (GEN && !inner)
+                    gh = *reinterpret_cast<const u64 *>(A.ghost + (2 * d + (left ? 0 : 1)) * A.nslots + vt * kWarp + c2);
 #pragma unroll
-                for (int d = 0; d < 3; d++) {  // W m_d: a power of two times an integer, exact
-                    const float4 M4 = *reinterpret_cast<const float4 *>(&sm.tab[b][d][kk]);
-                    wv[1 + d][0] = fmul2(pack2(W4.x, W4.y), pack2(M4.x, M4.y));
-                    wv[1 + d][1] = fmul2(pack2(W4.z, W4.w), pack2(M4.z, M4.w));
+                for (int k = 0; k < N1; k++) {
+                    u64 fl[N1], sv[N1], v[N1];
+#pragma unroll
+                    for (int j = 0; j < N1; j++) {
+                        fl[j] = f[row(k, j)];
+                        v[j] = ld2(&nbr[row(k, j)][c2]);
+                    }
+                    auto side = [&](auto left_c) {
+                        constexpr bool LEFT = decltype(left_c)::value;
+                        constexpr int R = LEFT ? 0 : N1 - 1;
+                        const u64 tj = trace_jump2<N1, LEFT>(v, fl[R], A.ops);
+                        const u64 tr = GEN == 0 ? tj : (inner ? tj : fsub2(gh, fl[R]));  // (per element: a select)
+                        line_sums_jump2<N1, LEFT>(sv, fl, tr, A.ops);
+                    };
+                    if (left)
+                        side(std::true_type{});
+                    else
+                        side(std::false_type{});
+#pragma unroll
+                    for (int j = 0; j < N1; j++)
+                        acc[row(k, j)] = ffma2(cdir[d], sv[j], acc[row(k, j)]);
+                }
+            };
+            wait(bX);
+            lines(std::integral_constant<int, 0>{}, enx, pX, [](int k, int j) { return j + N1 * k; });
+            __syncwarp();  // the x-neighbour is consumed: the next tile's f_s
+            if (more && role && op == 0) {
+                fence_proxy_async();
+                issue(csrc, vl + 1, bX);
+            }
+            wait(bY);
+            lines(std::integral_constant<int, 1>{}, eny, pY, [](int k, int j) { return k + N1 * j; });
+            __syncwarp();  // the y-neighbour is consumed: the next tile's f^n
+            if (more && has_fn && role && op == 1) {
+                fence_proxy_async();
+                issue(csrc, vl + 1, bY);
+            }
+            // BGK source towards the conservative Maxwellian, Shu-Osher combination, store
+            float W0, W1;
+            unpack2(ld2(&sm.tab[b][3][c2]), W0, W1);
+            const float gm[2] = {W0 != 0.f ? 1.f : 0.f, W1 != 0.f ? 1.f : 0.f};  // the padding mask
+            const bool iso = !GEN || A.viso;
+            float mm[3][2], mms[2];
+#pragma unroll
+            for (int s = 0; s < 2; s++) {
+#pragma unroll
+                for (int d = 0; d < 3; d++)
+                    mm[d][s] = m[d][s] * m[d][s];
+                mms[s] = mm[0][s] + mm[1][s] + mm[2][s];
+                if (iso) {
+                    mm[0][s] = mm[1][s] = mms[s];
+                    mm[2][s] = 0.f;
                 }
             }
+            const u64 cg = pack2(A.kg * gm[0], A.kg * gm[1]), gm2 = pack2(gm[0], gm[1]);
+            float *dst = A.dst + fidx(vl, e, 0, c2, E, NQ);
+            auto put_out = [&](int q, u64 o) {  // the stored value, and its transposed copy for the moments
+                if (real)
+                    __stcs(reinterpret_cast<u64 *>(dst + q * kWarp), o);
+                st2(&F[row0 + q][c2 ^ (4 * ((q + (NQ % 8 ? NQ * hf : 0)) & 7))], o);  // (its row mod 8)
+            };
+            __syncwarp();  // every lane has read its rows of F
+            auto bgk_src = [&](auto vtau_c, auto lim_c) {
+                constexpr bool VT = decltype(vtau_c)::value, LIM = decltype(lim_c)::value;
 #pragma unroll
-            for (int r = 0; r < NR; r++) {
-                const int row = np + 8 * r;  // (row mod 8 = np)
-                const float4 v = *reinterpret_cast<const float4 *>(&F[row][kk ^ (4 * np)]);
-                const u64 v01 = pack2(v.x, v.y), v23 = pack2(v.z, v.w);
+                for (int q = 0; q < NQ; q++) {
+                    const float4 *pp = reinterpret_cast<const float4 *>(&sm.par[hf * Sm::kParElem + q * kParamStride]);
+                    const float4 pa = pp[0], pb = pp[1];  // (a, b_x, b_y, b_z), (p4, p5, p6, 2^x constant)
+                    float ex[2];
 #pragma unroll
-                for (int c = 0; c < 5; c++) {
-                    pm[r][c] = ffma2(wv[c][0], v01, pm[r][c]);
-                    pm[r][c] = ffma2(wv[c][1], v23, pm[r][c]);
+                    for (int s = 0; s < 2; s++) {
+                        const float lin = fmaf(pa.w, m[2][s], fmaf(pa.z, m[1][s], fmaf(pa.y, m[0][s], pa.x)));
+                        ex[s] = GEN ? fmaf(pb.x, mm[0][s], fmaf(pb.y, mm[1][s], fmaf(pb.z, mm[2][s], lin)))
+                                    : fmaf(pb.x, mms[s], fmaf(pb.y, mms[s], lin));
+                    }
+                    float g[2];
+                    exp2_fp32x2(pack2(ex[0], ex[1]), dup2(pb.w), g[0], g[1]);
+                    u64 gc = cg;
+                    if constexpr (VT)  // kg = b - kb exactly, kb as in the accumulator above
+                        gc = fmul2(dup2(__fsub_rn(A.b, __fsub_rn(A.b, __fmul_rn(bdt, pb.z)))), gm2);
+                    acc[q] = ffma2(gc, pack2(g[0], g[1]), acc[q]);
+                    if constexpr (!LIM)
+                        put_out(q, acc[q]);
                 }
+            };
+            using T_ = std::true_type;
+            using F_ = std::false_type;
+            if constexpr (GEN) {
+                if (A.limiter)
+                    A.vtau ? bgk_src(T_{}, T_{}) : bgk_src(F_{}, T_{});
+                else
+                    A.vtau ? bgk_src(T_{}, F_{}) : bgk_src(F_{}, F_{});
+            } else {
+                bgk_src(F_{}, F_{});
             }
-        }
+            if (GEN && A.limiter) {
+                // Zhang-Shu (Sec. 2.1, Eqs. 10-11): the element mean (tensor Gauss-Legendre weights / 4, summing to
+                // 1) and minimum of each velocity, all in this lane's registers
+                u64 mean2 = 0;
+                float mn[2] = {3.4e38f, 3.4e38f}, mean[2];
 #pragma unroll
-        for (int r = 0; r < NR; r++)
+                for (int q = 0; q < NQ; q++) {
+                    mean2 = ffma2(dup2(A.ops.wq[q % N1] * A.ops.wq[q / N1]), acc[q], mean2);
+                    float o[2];
+                    unpack2(acc[q], o[0], o[1]);
+                    mn[0] = fminf(mn[0], o[0]);
+                    mn[1] = fminf(mn[1], o[1]);
+                }
+                unpack2(mean2, mean[0], mean[1]);
+                float beta[2];
 #pragma unroll
-            for (int c = 0; c < 5; c++)
-                msum[r][c] += sum2(pm[r][c]);
-        __syncwarp();  // this tile's f_s buffer is done with: the next tile's y-neighbour
-        if (more && role && op == 3) {
-            fence_proxy_async();
-            issue(nsrc, vl + 1, bF);
-        }
-        if (vl + 1 == ge) {  // the end of a moment group: combine the 4 velocity eighths of a row
-            const int grp = moment_group(A, unit / EB, vl);
-            ge = min(ge + A.G, vl1);
+                for (int s = 0; s < 2; s++)
+                    beta[s] = fminf(fabsf(mean[s] / (mean[s] - mn[s])), 1.f);
+                if (mn[0] < 0.f || mn[1] < 0.f) {
+#pragma unroll
+                    for (int q = 0; q < NQ; q++) {
+                        float o[2];
+                        unpack2(acc[q], o[0], o[1]);
+#pragma unroll
+                        for (int s = 0; s < 2; s++)
+                            o[s] = mn[s] < 0.f ? fmaf(beta[s], o[s] - mean[s], mean[s]) : o[s];
+                        acc[q] = pack2(o[0], o[1]);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < NQ; q++)
+                    put_out(q, acc[q]);
+            }
+            // moments of the elements' nodes (Eq. 2 with Eq. 12) of the stored values
+            __syncwarp();
+            u64 pm[NR][5];
 #pragma unroll
             for (int r = 0; r < NR; r++)
 #pragma unroll
-                for (int c = 0; c < 5; c++) {
-                    float s = msum[r][c];
-                    s += __shfl_xor_sync(0xffffffffu, s, 1);
-                    s += __shfl_xor_sync(0xffffffffu, s, 2);
-                    const int row = np + 8 * r;  // rows of the repeated half of an odd count: not stored
-                    if (kg == 0 && eb + row / NQ < E)
-                        A.partial[((int64_t)grp * 5 + c) * A.npts + (int64_t)eb * NQ + row] = s;
-                    msum[r][c] = 0.f;
+                for (int c = 0; c < 5; c++)
+                    pm[r][c] = 0ull;
+#pragma unroll
+            for (int k = 0; k < 8; k += 4) {
+                const int kk = 8 * kg + k;
+                u64 wv[5][2];
+                {
+                    const float4 W4 = *reinterpret_cast<const float4 *>(&sm.tab[b][3][kk]);
+                    const float4 E4 = *reinterpret_cast<const float4 *>(&sm.tab[b][4][kk]);
+                    wv[0][0] = pack2(W4.x, W4.y);
+                    wv[0][1] = pack2(W4.z, W4.w);
+                    wv[4][0] = pack2(E4.x, E4.y);
+                    wv[4][1] = pack2(E4.z, E4.w);
+#pragma unroll
+                    for (int d = 0; d < 3; d++) {  // W m_d: a power of two times an integer, exact
+                        const float4 M4 = *reinterpret_cast<const float4 *>(&sm.tab[b][d][kk]);
+                        wv[1 + d][0] = fmul2(pack2(W4.x, W4.y), pack2(M4.x, M4.y));
+                        wv[1 + d][1] = fmul2(pack2(W4.z, W4.w), pack2(M4.z, M4.w));
+                    }
                 }
+#pragma unroll
+                for (int r = 0; r < NR; r++) {
+                    const int row = np + 8 * r;  // (row mod 8 = np)
+                    const float4 v = *reinterpret_cast<const float4 *>(&F[row][kk ^ (4 * np)]);
+                    const u64 v01 = pack2(v.x, v.y), v23 = pack2(v.z, v.w);
+#pragma unroll
+                    for (int c = 0; c < 5; c++) {
+                        pm[r][c] = ffma2(wv[c][0], v01, pm[r][c]);
+                        pm[r][c] = ffma2(wv[c][1], v23, pm[r][c]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < NR; r++)
+#pragma unroll
+                for (int c = 0; c < 5; c++)
+                    msum[r][c] += sum2(pm[r][c]);
+            __syncwarp();  // this tile's f_s buffer is done with: the next tile's y-neighbour
+            if (more && role && op == 3) {
+                fence_proxy_async();
+                issue(nsrc, vl + 1, bF);
+            }
+            if (turn) {
+                csrc = nsrc;
+                octc = octn;
+                enx = upwind_neighbour(A.mesh, ec, 0, (octc & 1) != 0);
+                eny = upwind_neighbour(A.mesh, ec, 1, (octc & 2) != 0);
+            }
+            const int t = bF;
+            bF = bX;
+            bX = bN;
+            bN = bY;
+            bY = t;
         }
-        if (turn) {
-            csrc = nsrc;
-            octc = octn;
-            enx = upwind_neighbour(A.mesh, ec, 0, (octc & 1) != 0);
-            eny = upwind_neighbour(A.mesh, ec, 1, (octc & 2) != 0);
-        }
-        const int t = bF;
-        bF = bX;
-        bX = bN;
-        bN = bY;
-        bY = t;
+        // the end of a moment group: combine the 4 velocity eighths of a row
+        const int grp = moment_group(A, unit / EB, vl - 1);
+        ge = min(ge + A.G, vl1);
+#pragma unroll
+        for (int r = 0; r < NR; r++)
+#pragma unroll
+            for (int c = 0; c < 5; c++) {
+                float s = msum[r][c];
+                s += __shfl_xor_sync(0xffffffffu, s, 1);
+                s += __shfl_xor_sync(0xffffffffu, s, 2);
+                const int row = np + 8 * r;  // rows of the repeated half of an odd count: not stored
+                if (kg == 0 && eb + row / NQ < E)
+                    A.partial[((int64_t)grp * 5 + c) * A.npts + (int64_t)eb * NQ + row] = s;
+                msum[r][c] = 0.f;
+            }
     }
 }
 

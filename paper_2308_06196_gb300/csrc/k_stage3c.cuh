@@ -683,21 +683,21 @@ __global__ void __launch_bounds__(kWarp *N1, (N1 >= 4 ? BGK_STAGE3C_MINCTAS_P3 :
             }
             ka = ka == 2 ? 0 : ka + 1;
         }
-            const int grp = moment_group(A, blockIdx.x / E, vl - 1);
+        const int grp = moment_group(A, blockIdx.x / E, vl - 1);
 #pragma unroll
-            for (int h = 0; h < NHR; h++) {
-                const int q = np + 8 * h;
+        for (int h = 0; h < NHR; h++) {
+            const int q = np + 8 * h;
 #pragma unroll
-                for (int c = 0; c < 5; c++) {
-                    float x = msum[h][c];
-                    msum[h][c] = 0.f;
-                    x += __shfl_xor_sync(0xffffffffu, x, 1);
-                    x += __shfl_xor_sync(0xffffffffu, x, 2);
-                    if (kg == 0 && q < NQ)
-                        A.partial[((int64_t)grp * 5 + c) * A.npts + (int64_t)e * NP + q + NQ * w] = x;
-                }
+            for (int c = 0; c < 5; c++) {
+                float x = msum[h][c];
+                msum[h][c] = 0.f;
+                x += __shfl_xor_sync(0xffffffffu, x, 1);
+                x += __shfl_xor_sync(0xffffffffu, x, 2);
+                if (kg == 0 && q < NQ)
+                    A.partial[((int64_t)grp * 5 + c) * A.npts + (int64_t)e * NP + q + NQ * w] = x;
             }
-            ge = min(ge + A.G, vl1);
+        }
+        ge = min(ge + A.G, vl1);
     }
 }
 

@@ -475,21 +475,21 @@ __global__ void __launch_bounds__(kWarp *BGK_STAGE3W_WARPS, (N1 == 3 ? BGK_STAGE
             ka = ka == 2 ? 0 : ka + 1;
         }
         // the end of a moment group: combine the 4 velocity eighths of every row
-            const int grp = moment_group(A, blockIdx.x / nblk, vl - 1);
+        const int grp = moment_group(A, blockIdx.x / nblk, vl - 1);
 #pragma unroll
-            for (int h = 0; h < NHR; h++) {
-                const int q = np + 8 * h;
+        for (int h = 0; h < NHR; h++) {
+            const int q = np + 8 * h;
 #pragma unroll
-                for (int c = 0; c < 5; c++) {
-                    float x = msum[h][c];
-                    msum[h][c] = 0.f;
-                    x += __shfl_xor_sync(0xffffffffu, x, 1);
-                    x += __shfl_xor_sync(0xffffffffu, x, 2);
-                    if (kg == 0 && q < NP)
-                        A.partial[((int64_t)grp * 5 + c) * A.npts + (int64_t)e * NP + q] = x;
-                }
+            for (int c = 0; c < 5; c++) {
+                float x = msum[h][c];
+                msum[h][c] = 0.f;
+                x += __shfl_xor_sync(0xffffffffu, x, 1);
+                x += __shfl_xor_sync(0xffffffffu, x, 2);
+                if (kg == 0 && q < NP)
+                    A.partial[((int64_t)grp * 5 + c) * A.npts + (int64_t)e * NP + q] = x;
             }
-            ge = min(ge + A.G, vl1);
+        }
+        ge = min(ge + A.G, vl1);
     }
 }
 
