@@ -331,7 +331,7 @@ __device__ __forceinline__ void line_task(const StageArgs &A, const int task, co
 // exponents (a shared load returns 128 bytes per cycle, broadcast or not) once per 64 velocities. f_s is
 // double-buffered between the rows of the run's two outside neighbours (only the upwind one is copied), f^n
 // single (the next tile's lands once this tile's is in registers). Bound: latency and issue at 12 warps per SM.
-// 65,536 elements at p = 3, 32^2 velocities: 0.147 -> 0.121 ms per octant launch (5.9 TB/s); 60,001 at p = 1,
+// 65,536 elements at p = 3, 32^2 velocities: 0.148 -> 0.127 ms per octant launch (5.7 TB/s); 60,001 at p = 1,
 // 40^2 velocities, three steps 7.78 -> 4.02 ms; four steps of the Sod ensemble with their sampling 26.7 -> 24.8.
 // ------------------------------------------------------------------------------------------------
 template <int N1>
