@@ -29,7 +29,6 @@ cudaError_t launch_newton_batch(const NewtonArgs *d_args, const int *d_pt_start,
 cudaError_t launch_stage1d_batch(int n1, const StageArgs *d_args, const int2 *d_task_member, int *d_block,
                                  int ctas, cudaStream_t s);
 cudaError_t set_batch_ops(int n1, const Ops &op);
-int stage1d_tasks(const StageArgs &A);
 int stage1d_batch_tasks(const StageArgs &A);
 int stage1d_batch_ctas(int n1);
 cudaError_t launch_init_maxwellian(float *f, const double *prim, const float *mi, const float *gmask, int nslots,
@@ -1938,6 +1937,17 @@ int bfail(bgk_batch *b, int code, const std::string &msg)
             return bfail(b, BGK_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
+// Member c's stage arguments in a batch (the caller sets the buffers and the step): its one chunk, in tasks of
+// at least kBatchTiles tiles unless its length was given or measured. The task table and bgk_batch_info both count
+// these tasks.
+StageArgs batch_member_args(bgk_ctx *c)
+{
+    StageArgs A = stage_args(c, c->chunks[0]);
+    A.R = A.fixed ? 1 : std::max(1, kBatchTiles / A.G);
+    A.ntasks = (A.ngroups + A.R - 1) / A.R;
+    return A;
+}
+
 // Build and upload the members' stage and Newton arguments for time steps dt (one chunk per member:
 // stage 1 A -> slot 0, stage 2 slot 0 (+ A) -> slot 1, stage 3 slot 1 (+ A) -> A in place).
 int batch_upload(bgk_batch *b, const double *dt)
@@ -1950,15 +1960,12 @@ int batch_upload(bgk_batch *b, const double *dt)
         b->alg_bytes[s] = 0.0;
     for (int q = 0; q < n; q++) {
         bgk_ctx *c = b->probs[q];
-        const Chunk &ch = c->chunks[0];
         float *Aq = c->fA, *s1 = c->pool, *s2 = c->pool + c->chunk_floats;
         int64_t real = 0;
         for (int v = 0; v < c->nslots; v++)
             real += c->slotk[v] >= 0;
         for (int st = 0; st < 3; st++) {
-            StageArgs A = stage_args(c, ch);
-            A.R = A.fixed ? 1 : std::max(1, kBatchTiles / A.G);
-            A.ntasks = (A.ngroups + A.R - 1) / A.R;
+            StageArgs A = batch_member_args(c);
             A.src = st == 0 ? Aq : (st == 1 ? s1 : s2);
             A.fn = st == 0 ? nullptr : Aq;
             A.dst = st == 0 ? s1 : (st == 1 ? s2 : Aq);
@@ -2334,7 +2341,7 @@ int bgk_batch_info(const bgk_batch *b, int64_t *npoints, int64_t *ndof, int64_t 
     for (const bgk_ctx *c : b->probs) {
         np += c->npts;
         nd += c->npts * c->nvel;
-        nt += stage1d_tasks(stage_args(const_cast<bgk_ctx *>(c), c->chunks[0]));
+        nt += stage1d_batch_tasks(batch_member_args(const_cast<bgk_ctx *>(c)));
     }
     if (npoints)
         *npoints = np;

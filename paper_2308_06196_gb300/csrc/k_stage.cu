@@ -703,18 +703,6 @@ static void plan_line(StageArgs &A)
     plan_tasks(A, (A.mesh.nelem + K - 1) / K, 152 * BGK_LINE_MINCTAS * BGK_LINE_WARPS, 0.8, 0.6);
 }
 
-int stage1d_tasks(const StageArgs &A)
-{
-    switch (A.n1) {
-    case 2: return line_tasks<2>(A);
-    case 3: return line_tasks<3>(A);
-    case 4: return line_tasks<4>(A);
-    case 5: return line_tasks<5>(A);
-    case 6: return line_tasks<6>(A);
-    }
-    return 0;
-}
-
 __device__ __forceinline__ void line_init_barriers(uint32_t bar0)
 {
     if ((threadIdx.x & 31) == 0) {

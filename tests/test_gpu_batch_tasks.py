@@ -1,0 +1,50 @@
+"""The task count that a batch reports is the one that its stage launches share out: runs of two half-warps'
+elements (16 / (p + 1) each) times tasks of whole moment groups, at least 16 tiles long unless the length was
+given or measured."""
+import pytest
+
+from paper_2308_06196_gb300 import _build, workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def tiles(nv):
+    """32-velocity tiles of a grid that is symmetric about 0: the octants are padded one by one."""
+    n = 0
+    for o in range(8):
+        side = [k // 2 if not (o >> d) & 1 else k - k // 2 for d, k in enumerate(nv)]
+        n += -(-side[0] * side[1] * side[2] // 32)
+    return n
+
+
+def count(m, G):
+    """Tasks of member m with groups of G tiles; G = 0: the library's own groups and task length."""
+    nvt, E = tiles(m["nv"]), m["nelem"][0]
+    R = 1
+    if G == 0:
+        G = max(1, min(8, nvt * E // (152 * 32)))
+        R = max(1, 16 // G)
+    run = 2 * (16 // (m["p"] + 1))
+    return -(-E // run) * -(-(-(-nvt // G)) // R)
+
+
+@pytest.mark.parametrize("G", [0, 1, 3, 32])
+def test_reported_tasks(G):
+    _build.build()
+    from paper_2308_06196_gb300.bgk import Batch, Solver
+
+    ms = W.sod_members(members=7, seed=3, elements=(5, 400), degrees=(1, 3), nvs=(12, 15, 24))
+    k = [W.mesh_kwargs(m) for m in ms]
+    ss = [Solver(c["dim"], c["nelem"], c["lo"], c["hi"], c["p"], c["nv"], c["vlo"], c["vhi"], c["tau"], bc=m["bc"],
+                 bc_state=m["bc_state"], chunks=1, vtiles_per_task=G) for c, m in zip(k, ms)]
+    for s, m in zip(ss, ms):
+        s.set_state(W.prim_sod(s.points(), m["left"], m["right"]))
+    b = Batch(ss)
+    assert b.tasks == sum(count(c, G) for c in k)
+    b.step([s.dt(0.1) for s in ss], 1)
+    b.synchronize()
+    one = Batch(ss[:1])
+    one.autotune()  # a measured length: one group per task, of one of the candidates
+    nvt = tiles(k[0]["nv"])
+    cands = [2, 4, 8, 16, 32, 64] + [-(-nvt // q) for q in (1, 2, 3, 4, 6, 8, 12, 16)]
+    assert one.tasks in {count(k[0], g) for g in cands if 2 <= g <= 64}
