@@ -596,7 +596,7 @@ int enqueue_step64(bgk_ctx *c, double dt, cudaStream_t s)
             if (rc)
                 return rc;
         }
-        CK(launch_table64(c->etab64, c->par64, table64_args(c), (int)c->npts, s));
+        bool tabled = false;
         for (const Launch &l : stage_launches(c)) {
             double *Aq = chunk_ptr64(c, c->fA64, l.vt0);
             double *s1 = c->pool64 + pool_offset(c, l.chunk, 0);
@@ -635,6 +635,9 @@ int enqueue_step64(bgk_ctx *c, double dt, cudaStream_t s)
             A.fbase = c->fbase;
             A.rhowu = c->rhowu64;
             ev_begin(c, 0, (double)l.real * c->npts * sizeof(double) * (st == 0 ? 2 : 3));
+            if (!tabled)  // the Maxwellian's factors of all chunks: part of the stage's time
+                CK(launch_table64(c->etab64, c->par64, table64_args(c), (int)c->npts, s));
+            tabled = true;
             CK(launch_stage64(A, s));
             if (c->opts.limiter)
                 CK(launch_limit64(A.dst, A.nvt, c->E, c->NP, c->N1, c->dim, c->ops64, c->ijac64, s));
