@@ -11,6 +11,7 @@
 // A stage reads neighbours only inside its own chunk, and chunks run in order on one stream, so a
 // slot is rewritten only after the launch that read it has finished. Memory = A + (C+1)/C arrays.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -58,6 +59,21 @@ const double kPi = 3.14159265358979323846;
 // Stage buffers up to this size are kept in full (two f arrays instead of one and a chunk), so that the
 // chunks of a stage can go in one launch (see bgk_create)
 const int64_t kMergeBytes = 64ll << 20;
+// What all contexts of the process may hold together for that beyond the rotating slots: a program that fills
+// the device with small contexts loses 0.4 % of it at most; the contexts past this step chunk by chunk (the same
+// results, 1.1 to 2.2 times the time per step when alone on the chip: see bgk_create)
+const int64_t kMergeExtra = 1ll << 30;
+std::atomic<int64_t> g_merge_extra{0};
+
+bool reserve_merge_extra(int64_t bytes)
+{
+    int64_t held = g_merge_extra.load();
+    do {
+        if (held + bytes > kMergeExtra)
+            return false;
+    } while (!g_merge_extra.compare_exchange_weak(held, held + bytes));
+    return true;
+}
 // Tiles per task of the batched line launches (whole moment groups of at least this, see batch_upload)
 #ifndef BGK_BATCH_TILES
 #define BGK_BATCH_TILES 16
@@ -201,6 +217,7 @@ struct bgk_ctx {
     int64_t chunk_floats = 0;  // floats per pool slot
     bool task_fixed = false;   // G is the task length too (chosen by the user or the autotuner)
     bool merged = false;       // small problem: one launch per stage over all chunks, two full stage buffers
+    int64_t merge_extra = 0;   // bytes reserved of kMergeExtra for them
     // device buffers
     float *fA = nullptr, *pool = nullptr;
     float *xi = nullptr, *mi = nullptr, *wpsi = nullptr, *gmask = nullptr, *ghost = nullptr;
@@ -749,6 +766,7 @@ void bgk_destroy(bgk_ctx *c)
     for (void *b : bufs)
         if (b)
             cudaFree(b);
+    g_merge_extra -= c->merge_extra;  // (after the buffers' release)
     if (c->own)
         cudaStreamDestroy(c->own);
     delete c;
@@ -954,8 +972,8 @@ int bgk_create(const bgk_mesh *mesh, int p, const bgk_vgrid *vg, double tau, con
 
     // Small problems: all chunks of a stage in one launch. A stage of a few microseconds per chunk is bound by
     // the launches and by their nearly empty chip (a 24-element shock tube, 12^3 velocities, 20 steps with a
-    // checkpoint: 3.42 -> 1.80 ms; 3 x 2 x 4 elements at p = 3, 14^3 velocities, 17 MB of f: 0.43 -> 0.34 ms
-    // per pass); above the limit the octants' own kernels and the smaller memory win.
+    // checkpoint: 3.42 -> 1.80 ms; per step, chunk by chunk -> together: that tube 152 -> 70 us, 3 x 2 x 4 elements
+    // at p = 3, 14^3 velocities, 16 MB of f, 215 -> 129, 5 x 4 x 4 elements, 54 MB, 334 -> 276); above the limit the octants' own kernels and the smaller memory win.
     const int64_t fA = (int64_t)c->nvt * E * c->NP * kWarp;
     c->merged = c->opts.chunks == 0 && c->chunks.size() > 1 && fA * c->esize <= kMergeBytes;
     // memory check before any allocation
@@ -963,16 +981,18 @@ int bgk_create(const bgk_mesh *mesh, int p, const bgk_vgrid *vg, double tau, con
                            (int64_t)c->nslots * 4 * 25 +
                            (c->prec == BGK_FP64 ? c->npts * 8 * (c->nv[0] + c->nv[1] + c->nv[2]) : 0) +
                            (c->has_exchange ? 2 * (int64_t)c->nvt * c->ne[1] * c->ne[2] * c->NP * kWarp * 4 : 0);
-    int64_t pool = c->merged ? 2 * fA : (int64_t)(c->chunks.size() + 1) * c->chunk_floats;
-    int64_t need = (fA + pool) * c->esize + tables;
+    const int64_t slots = (int64_t)(c->chunks.size() + 1) * c->chunk_floats;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess)
         return bail(BGK_ECUDA, "cudaMemGetInfo failed (no CUDA device?)");
-    if (c->merged && (double)need > 0.97 * (double)free_b) {  // the two full buffers do not fit: chunk by chunk
-        c->merged = false;
-        pool = (int64_t)(c->chunks.size() + 1) * c->chunk_floats;
-        need = (fA + pool) * c->esize + tables;
+    if (c->merged) {  // where the two full buffers do not fit, or other contexts hold what there is for them:
+        // chunk by chunk
+        const int64_t extra = std::max<int64_t>(0, (2 * fA - slots) * c->esize);
+        c->merged = (double)(3 * fA * c->esize + tables) <= 0.97 * (double)free_b && reserve_merge_extra(extra);
+        c->merge_extra = c->merged ? extra : 0;
     }
+    const int64_t pool = c->merged ? 2 * fA : slots;
+    const int64_t need = (fA + pool) * c->esize + tables;
     if ((double)need > 0.97 * (double)free_b)
         return bail(BGK_ENOMEM, "configuration needs " + std::to_string(need >> 20) + " MiB, only " +
                                     std::to_string(free_b >> 20) + " MiB free");
