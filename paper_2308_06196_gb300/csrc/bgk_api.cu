@@ -1822,7 +1822,7 @@ int bgk_autotune(bgk_ctx *c, int *g_out)
     snprintf(key, sizeof key, "%d/%d/%d,%d,%d/%d,%d,%d/%zu/%d", c->dim, c->p, c->nv[0], c->nv[1], c->nv[2], c->ne[0],
              c->ne[1], c->ne[2], c->chunks.size(),
              (int)(c->has_wall || c->has_force || c->bc[0] || c->bc[2] || c->bc[4]) + 2 * (c->met != nullptr) +
-                 4 * (c->ftab != nullptr));
+                 4 * (c->ftab != nullptr) + 8 * c->merged);
     for (auto &kv : g_tuned)
         if (kv.first == key) {
             set_task_length(c, kv.second);
