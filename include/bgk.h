@@ -93,7 +93,12 @@ typedef struct {
     int limiter;             /* 1: Zhang-Shu positivity limiter (Sec. 2.1, Eqs. 10-11) on every stage output,
                                 per element and velocity: towards the Gauss-Legendre-weighted element mean
                                 where a node value is negative. Keeps element means (so conservation). */
-    int chunks;              /* velocity chunks per stage, 0 = automatic */
+    int chunks;              /* velocity chunks per stage. 1: all velocities in one chunk. Otherwise one chunk per
+                                sign octant of the velocity grid: 0 (automatic) launches the chunks of a stage
+                                together where f takes at most 64 MB (with two full stage buffers, of which all
+                                contexts together hold at most 1 GiB beyond the rotating ones) and one after
+                                the other on rotating buffers elsewhere; any other value always one after the
+                                other. The results do not depend on how the octants are launched. */
     int vtiles_per_task;     /* 32-velocity tiles per warp task, 0 = automatic */
     int maxwellian;          /* BGK_MAXWELLIAN_CONSERVATIVE (0, the method) or BGK_MAXWELLIAN_CONTINUOUS
                                 (the ablation: g = the sampled continuous Maxwellian of the moments, whose
