@@ -48,3 +48,34 @@ def test_reported_tasks(G):
     nvt = tiles(k[0]["nv"])
     cands = [2, 4, 8, 16, 32, 64] + [-(-nvt // q) for q in (1, 2, 3, 4, 6, 8, 12, 16)]
     assert one.tasks in {count(k[0], g) for g in cands if 2 <= g <= 64}
+
+
+@pytest.mark.parametrize("G", [0, 1, 5])
+def test_batch_equals_members_alone_bit_for_bit(G):
+    """The batch shares the same moment groups out in tasks of its own length."""
+    import numpy as np
+
+    _build.build()
+    from paper_2308_06196_gb300.bgk import Batch, Solver
+
+    ms = W.sod_members(members=9, seed=8, elements=(5, 90), degrees=(1, 3), nvs=(12, 15, 24))
+
+    def make():
+        out = []
+        for m in ms:
+            c = W.mesh_kwargs(m)
+            s = Solver(c["dim"], c["nelem"], c["lo"], c["hi"], c["p"], c["nv"], c["vlo"], c["vhi"], c["tau"], bc=m["bc"],
+                       bc_state=m["bc_state"], chunks=1, vtiles_per_task=G)
+            s.set_state(W.prim_sod(s.points(), m["left"], m["right"]))
+            out.append(s)
+        return out
+
+    alone, members = make(), make()
+    dt = [s.dt(0.1) for s in alone]
+    b = Batch(members)
+    b.step(dt, 3)
+    b.synchronize()
+    for s, t, h in zip(alone, members, dt):
+        s.step(h, 3)
+        for x, y in ((s.moments(), t.moments()), (s.equilibrium(), t.equilibrium()), (s.get_f(), t.get_f())):
+            assert np.array_equal(x, y)
