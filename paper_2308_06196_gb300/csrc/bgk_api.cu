@@ -43,7 +43,7 @@ cudaError_t launch_limit64(double *f, int nvt, int E, int NP, int N1, int dim, c
 cudaError_t launch_wall(const WallArgs &A, bool fp64, const void *w, const void *xi, cudaStream_t s);
 cudaError_t launch_moments64(const Moments64Args &A, cudaStream_t s);
 cudaError_t launch_init64(double *f, const double *prim, double *par, double *tab, const Table64Args &T,
-                          const float *gmask, int nvt, int npts, int vdim, int *err, cudaStream_t s);
+                          const float *gmask, int nvt, int npts, int block, int vdim, int *err, cudaStream_t s);
 cudaError_t launch_table64(double *tab, const double *par, const Table64Args &T, int npts, cudaStream_t s);
 cudaError_t launch_convert64(bool to_device, double *f, double *st, const int *slotk, int nvt, int E, int NP,
                              int64_t nvel, int p0, int npt, cudaStream_t s);
@@ -228,7 +228,8 @@ struct bgk_ctx {
     // all-FP64 form
     int prec = BGK_FP32_SPLIT;
     double *fA64 = nullptr, *pool64 = nullptr, *xi64 = nullptr, *wpsi64 = nullptr, *ghost64 = nullptr, *par64 = nullptr;
-    double *etab64 = nullptr;  // [n_x][sum_d n_d] 1-D factors of the Maxwellian (all-FP64 form)
+    double *etab64 = nullptr;  // [eblock64 NP][sum_d n_d] 1-D factors of the Maxwellian (all-FP64 form)
+    int eblock64 = 0;          // elements whose factors it holds: all, or as many as the memory leaves room for
     // diffuse walls and body force
     bool has_wall = false, has_force = false;
     // exchange faces (x faces shared with a neighbouring subdomain): the halos, [nvt][E_face][NP][32]
@@ -652,10 +653,15 @@ int enqueue_step64(bgk_ctx *c, double dt, cudaStream_t s)
             A.fbase = c->fbase;
             A.rhowu = c->rhowu64;
             ev_begin(c, 0, (double)l.real * c->npts * sizeof(double) * (st == 0 ? 2 : 3));
-            if (!tabled)  // the Maxwellian's factors of all chunks: part of the stage's time
-                CK(launch_table64(c->etab64, c->par64, table64_args(c), (int)c->npts, s));
-            tabled = true;
-            CK(launch_stage64(A, s));
+            for (int64_t e0 = 0; e0 < c->E; e0 += c->eblock64) {
+                A.e0 = (int)e0;
+                A.ecount = (int)std::min<int64_t>(c->eblock64, c->E - e0);
+                // the Maxwellian's factors: once per stage for all chunks, where the table holds all elements
+                if (!tabled)
+                    CK(launch_table64(c->etab64, c->par64 + e0 * c->NP * 5, A.tab, A.ecount * c->NP, s));
+                tabled = c->eblock64 == c->E;
+                CK(launch_stage64(A, s));
+            }
             if (c->opts.limiter)
                 CK(launch_limit64(A.dst, A.nvt, c->E, c->NP, c->N1, c->dim, c->ops64, c->ijac64, s));
             ev_end(c);
@@ -979,16 +985,17 @@ int bgk_create(const bgk_mesh *mesh, int p, const bgk_vgrid *vg, double tau, con
     // memory check before any allocation
     const int64_t tables = (int64_t)c->max_groups * 5 * c->npts * 4 + c->npts * (5 * 8 * 3 + kParamStride * 4) +
                            (int64_t)c->nslots * 4 * 25 +
-                           (c->prec == BGK_FP64 ? c->npts * 8 * (c->nv[0] + c->nv[1] + c->nv[2]) : 0) +
                            (c->has_exchange ? 2 * (int64_t)c->nvt * c->ne[1] * c->ne[2] * c->NP * kWarp * 4 : 0);
     const int64_t slots = (int64_t)(c->chunks.size() + 1) * c->chunk_floats;
+    // the factors of one element's Maxwellians (all-FP64 form)
+    const int64_t row64 = c->prec == BGK_FP64 ? (int64_t)c->NP * 8 * (c->nv[0] + c->nv[1] + c->nv[2]) : 0;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess)
         return bail(BGK_ECUDA, "cudaMemGetInfo failed (no CUDA device?)");
     if (c->merged) {  // where the two full buffers do not fit, or other contexts hold what there is for them:
         // chunk by chunk
         const int64_t extra = std::max<int64_t>(0, (2 * fA - slots) * c->esize);
-        c->merged = (double)(3 * fA * c->esize + tables) <= 0.97 * (double)free_b && reserve_merge_extra(extra);
+        c->merged = (double)(3 * fA * c->esize + tables + 2 * E * row64) <= 0.97 * (double)free_b && reserve_merge_extra(extra);
         c->merge_extra = c->merged ? extra : 0;
     }
     const int64_t pool = c->merged ? 2 * fA : slots;
@@ -996,6 +1003,11 @@ int bgk_create(const bgk_mesh *mesh, int p, const bgk_vgrid *vg, double tau, con
     if ((double)need > 0.97 * (double)free_b)
         return bail(BGK_ENOMEM, "configuration needs " + std::to_string(need >> 20) + " MiB, only " +
                                     std::to_string(free_b >> 20) + " MiB free");
+    // the table of factors takes 3 / n^2 of f on n^3 velocities but up to an eighth on a grid with one long axis:
+    // where that is more than half of what is left (a geometry may follow), it holds some of the elements at a time
+    if (row64)
+        c->eblock64 = (int)std::max<int64_t>(
+            1, std::min<int64_t>(E, (int64_t)(0.5 * (0.97 * (double)free_b - (double)need)) / row64));
     for (int q = 0; q < 6; q++)
         if (q / 2 < c->dim && c->bc[q] == BGK_BC_DIRICHLET && !(c->bcs[q * 5] > 0.0 && c->bcs[q * 5 + 4] > 0.0))
             return bail(BGK_EINVAL, "Dirichlet state needs rho > 0 and T > 0");
@@ -1010,7 +1022,7 @@ int bgk_create(const bgk_mesh *mesh, int p, const bgk_vgrid *vg, double tau, con
         AL(c->wpsi64, 5 * c->nslots);
         AL(c->ghost64, 6 * c->nslots);
         AL(c->par64, c->npts * 5);
-        AL(c->etab64, c->npts * (c->nv[0] + c->nv[1] + c->nv[2]));
+        AL(c->etab64, (int64_t)c->eblock64 * c->NP * (c->nv[0] + c->nv[1] + c->nv[2]));
         if (c->opts.mu_ref > 0.0)
             AL(c->itau64, c->npts);
     } else {
@@ -1194,7 +1206,7 @@ static int set_state_impl(bgk_ctx *c, const double *prim, cudaMemcpyKind kind)
     CK(cudaMemcpyAsync(c->prim_in, prim, c->npts * 5 * sizeof(double), kind, c->stream));
     if (c->prec == BGK_FP64)
         CK(launch_init64(c->fA64, c->prim_in, c->par64, c->etab64, table64_args(c), c->gmask, c->nvt, (int)c->npts,
-                         c->vdim, c->err, c->stream));
+                         c->eblock64 * c->NP, c->vdim, c->err, c->stream));
     else
         CK(launch_init_maxwellian(c->fA, c->prim_in, c->mi, c->gmask, c->nslots, c->nvt, c->E, c->NP, c->nv, c->vlo,
                                   c->dv, c->err, c->Q, c->prim, c->stream));

@@ -221,7 +221,8 @@ struct Stage64Args {
     double *dst;
     const double *xi;      // [3][nslots]
     const double *ghost;   // [6][nslots]
-    const double *etab;    // [n_x][n_x-axis + n_y + n_z] the Maxwellian's 1-D factors (k64_table)
+    const double *etab;    // [ecount NP][n_x-axis + n_y + n_z] the Maxwellian's 1-D factors (k64_table)
+    int e0, ecount;        // elements of the launch
     Table64Args tab;
     const double *rhow;    // [6][nfmax][N1^2] diffuse-wall densities, or null
     const double *fpar;    // [n_x][5] body-force polynomial, or null

@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kWarp) k64_stage(const Stage64Args A)
 {
     extern __shared__ double acc64[];  // [NP][32]
     const int NP = A.NP, E = A.mesh.nelem, dim = A.mesh.dim, lane = threadIdx.x;
-    const int vl = blockIdx.x / E, e = blockIdx.x % E;
+    const int vl = blockIdx.x / A.ecount, el = blockIdx.x % A.ecount, e = A.e0 + el;
     const int slot = (A.vt0 + vl) * kWarp + lane;
     const int ec[3] = {e % A.mesh.ne[0], (e / A.mesh.ne[0]) % A.mesh.ne[1], e / (A.mesh.ne[0] * A.mesh.ne[1])};
     const int oct = A.toct[A.vt0 + vl];
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(kWarp) k64_stage(const Stage64Args A)
 #pragma unroll 4
     for (int i = 0; i < NP; i++) {
         const int64_t pt = (int64_t)e * NP + i;
-        const double *t = A.etab + pt * nt;
+        const double *t = A.etab + ((int64_t)el * NP + i) * nt;
         const double kg = bdt * (A.itau ? A.itau[pt] : A.inv_tau);
         double w = kg * gm;
         if (A.fpar) {  // body-force source g (q0 + q . xi + q4 |xi|^2)
@@ -228,16 +228,17 @@ __global__ void __launch_bounds__(kWarp) k64_stage(const Stage64Args A)
 __global__ void __launch_bounds__(256) k64_stage_curved(const Stage64Args A)
 {
     const int NP = A.NP, N1 = A.N1, E = A.mesh.nelem, nt = A.tab.n[0] + A.tab.n[1] + A.tab.n[2];
-    const int64_t n = (int64_t)A.nvt * E * NP * kWarp;
+    const int64_t n = (int64_t)A.nvt * A.ecount * NP * kWarp;
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
         const int lane = (int)(q % kWarp);
         const int i = (int)((q / kWarp) % NP);
-        const int e = (int)((q / ((int64_t)kWarp * NP)) % E);
-        const int vl = (int)(q / ((int64_t)kWarp * NP * E));
+        const int el = (int)((q / ((int64_t)kWarp * NP)) % A.ecount), e = A.e0 + el;
+        const int vl = (int)(q / ((int64_t)kWarp * NP * A.ecount));
+        const int64_t at = fidx(vl, e, i, lane, E, NP);
         const int slot = (A.vt0 + vl) * kWarp + lane;
         const int ec[3] = {e % A.mesh.ne[0], (e / A.mesh.ne[0]) % A.mesh.ne[1], e / (A.mesh.ne[0] * A.mesh.ne[1])};
         const int ic[3] = {i % N1, (i / N1) % N1, i / (N1 * N1)};
-        const double fs = A.src[q];
+        const double fs = A.src[at];
         double xi[3];
         for (int d = 0; d < 3; d++)
             xi[d] = A.xi[d * A.nslots + slot];
@@ -246,7 +247,7 @@ __global__ void __launch_bounds__(256) k64_stage_curved(const Stage64Args A)
         // conservative Maxwellian of this point, BGK relaxation and the Shu-Osher combination
         int col[3];
         columns64(A.tab, slot, col);
-        const double *t = A.etab + ((int64_t)e * NP + i) * nt;
+        const double *t = A.etab + ((int64_t)el * NP + i) * nt;
         const double g = A.gmask[slot] * (t[col[0]] * t[col[1]] * t[col[2]]);
         double src = (g - fs) * (A.itau ? A.itau[(int64_t)e * NP + i] : A.inv_tau);
         if (A.fpar) {  // body-force source g (q0 + q . xi + q4 |xi|^2)
@@ -255,8 +256,8 @@ __global__ void __launch_bounds__(256) k64_stage_curved(const Stage64Args A)
         }
         double out = A.b * (fs + A.dt * (R + src));
         if (A.fn)
-            out += A.an * A.fn[q];
-        A.dst[q] = out;
+            out += A.an * A.fn[at];
+        A.dst[at] = out;
     }
 }
 
@@ -301,19 +302,19 @@ __global__ void k64_init_par(double *par, const double *prim, int npts, int vdim
     p[4] = ok ? 0.5 / s[4] : 0.0;
 }
 
-// Sample every point's tabulated Maxwellian into the FP64 layout (3 operations per degree of freedom where
-// an exponential and a power each took some 30).
+// Sample the tabulated Maxwellians of points p0 .. p0 + np - 1 into the FP64 layout (3 operations per degree of
+// freedom where an exponential and a power each took some 30).
 __global__ void __launch_bounds__(256) k64_init(double *f, const double *etab, const Table64Args T, const float *gmask,
-                                                int nvt, int npts)
+                                                int nvt, int npts, int p0, int np)
 {
-    const int64_t n = (int64_t)nvt * npts;
+    const int64_t n = (int64_t)nvt * np;
     const int nt = T.n[0] + T.n[1] + T.n[2], lane = threadIdx.x & 31;
     for (int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; q < n; q += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        const int slot = (int)(q / npts) * kWarp + lane;
+        const int slot = (int)(q / np) * kWarp + lane;
         int col[3];
         columns64(T, slot, col);
-        const double *t = etab + (q % npts) * nt;
-        f[q * kWarp + lane] = gmask[slot] * (t[col[0]] * t[col[1]] * t[col[2]]);
+        const double *t = etab + (q % np) * nt;
+        f[((q / np) * npts + p0 + q % np) * kWarp + lane] = gmask[slot] * (t[col[0]] * t[col[1]] * t[col[2]]);
     }
 }
 
@@ -384,14 +385,14 @@ template <int N1>
 static cudaError_t stage64(const Stage64Args &A, cudaStream_t s)
 {
     const int smem = A.NP * kWarp * (int)sizeof(double);  // at most 16 KB (p = 3, 3-D)
-    k64_stage<N1><<<A.nvt * A.mesh.nelem, kWarp, smem, s>>>(A);
+    k64_stage<N1><<<A.nvt * A.ecount, kWarp, smem, s>>>(A);
     return cudaGetLastError();
 }
 
 cudaError_t launch_stage64(const Stage64Args &A, cudaStream_t s)
 {
     if (A.ja) {
-        k64_stage_curved<<<grid_for((int64_t)A.nvt * A.mesh.nelem * A.NP * kWarp, 256), 256, 0, s>>>(A);
+        k64_stage_curved<<<grid_for((int64_t)A.nvt * A.ecount * A.NP * kWarp, 256), 256, 0, s>>>(A);
         return cudaGetLastError();
     }
     switch (A.N1) {
@@ -415,18 +416,22 @@ cudaError_t launch_moments64(const Moments64Args &A, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// f sampled from prim: par and tab (the next solve's parameters and tables) hold the intermediate values.
+// f sampled from prim by blocks of at most `block` points, which tab holds: par and tab (the next solve's parameters and
+// tables) take the intermediate values.
 cudaError_t launch_init64(double *f, const double *prim, double *par, double *tab, const Table64Args &T,
-                          const float *gmask, int nvt, int npts, int vdim, int *err, cudaStream_t s)
+                          const float *gmask, int nvt, int npts, int block, int vdim, int *err, cudaStream_t s)
 {
     k64_init_par<<<(npts + 127) / 128, 128, 0, s>>>(par, prim, npts, vdim, err);
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess)
-        e = launch_table64(tab, par, T, npts, s);
-    if (e != cudaSuccess)
-        return e;
-    k64_init<<<grid_for((int64_t)nvt * npts * kWarp, 256), 256, 0, s>>>(f, tab, T, gmask, nvt, npts);
-    return cudaGetLastError();
+    for (int64_t p0 = 0; p0 < npts && e == cudaSuccess; p0 += block) {
+        const int np = (int)std::min<int64_t>(block, npts - p0);
+        e = launch_table64(tab, par + p0 * 5, T, np, s);
+        if (e != cudaSuccess)
+            break;
+        k64_init<<<grid_for((int64_t)nvt * np * kWarp, 256), 256, 0, s>>>(f, tab, T, gmask, nvt, npts, (int)p0, np);
+        e = cudaGetLastError();
+    }
+    return e;
 }
 
 cudaError_t launch_convert64(bool to_device, double *f, double *st, const int *slotk, int nvt, int E, int NP,
