@@ -115,13 +115,25 @@ struct StageArgs {
 // resident at a time. A task writes its running moment sums out at the end of every group, so the partial sums
 // do not depend on R. Longer tasks share the set-up and the first copies, which are not hidden behind the
 // task's own work (about `start` tiles' time); shorter ones leave less of the chip idle in the last round,
-// which takes idle + (1 - idle) x of a full one's time when it is filled to x. The rule takes the least of
+// which takes idle + (1 - idle) x of a full one's time when it is filled to x (kIdleFew with fewer than kRounds
+// rounds). The rule takes the least of
 //   (tiles + start per task) units / wave + what the last round wastes of a task's length;
-// start and idle are the kernel's, from sweeps of the task length (tiles per task: us per launch). k_stage3s:
-// 16^3 elements, 54 tiles, 8: 1150, 16: 1131, 32: 1124, 54: 1169; 315 elements, 42 tiles, 1: 107, 2: 95, 3: 91,
-// 4: 91, 6: 96, 11: 109; 90 elements, 23 tiles, 1: 32, 3: 28, 6: 37. k_stage3w: 2048 elements, 128 tiles, 8: 740,
-// 16: 700, 32: 692, 64: 745; 360 elements, 69 to 86 tiles, 2: 100, 4: 92, 8: 89, 12: 103, 16: 87, 22: 105.
-inline void plan_tasks(StageArgs &A, int64_t units, int64_t wave, double start, double idle)
+// beyond `free` tiles only tasks of which kRounds rounds are left count (with fewer, a longer task gains what the last
+// round may cost), and those of short groups that nearly fill one round. start, idle and free are the kernel's. Over
+// 805 shapes of all kernels (70 MB to 2.6 GB of f, 16^3 to 48^3 velocities) the rule takes 0.964 of the time of one
+// group per task, the best R of each shape 0.956; its worst are 1.14 (curved pairs, 90 elements, 128 tiles) and 1.08.
+// Without the limits it took 0.971, and up to 1.24 (walls at p = 2, 6 x 6 x 3 elements of 40^3 velocities, groups of 5
+// tiles: 87 us per launch in single groups, 102 in threes, 0.93 of a round; 10 x 16 x 12 at p = 1, 18^3 velocities: 43
+// and 51). What the limits leave out, mean time of its tasks against single groups: G = 8, 1.5 to 2 rounds 1.03, 2 to 3
+// 1.01, 3 to 4 1.01; what they keep: beyond 4 rounds 0.995 (channel, 16 rounds, 0.94), G <= 2 and 0.9 to 1 round 0.96.
+// Tiles per task: us per launch: k_stage3s, 16^3 elements, 54 tiles, 8: 1150, 16: 1131, 32: 1124, 54: 1169; 315
+// elements, 42 tiles, 1: 107, 2: 95, 3: 91, 4: 91, 6: 96, 11: 109. k_stage3w, 2048 elements,
+// 128 tiles, 8: 740, 16: 700, 32: 692, 64: 745. k_stage3c, 240 elements, 32 tiles, 1: 224, 2: 199, 4: 199, 6: 180, 8:
+// 195. k_stage1d, 1713 runs, 11 tiles, 7: 28.8, 11: 28.2. k_stage1d_pair, 1688 runs, 54 tiles, 8: 165, 16: 163, 24: 163, 48:
+// 166. k_stage2p, 2048 pairs of elements, 54 tiles, 8: 244, 16: 239, 24: 242, 32: 269. k_stage3cp, 2688 elements, 54 tiles,
+// 8: 207, 16: 205, 24: 211, 32: 224.
+constexpr double kRounds = 4.0, kIdleFew = 0.75;
+inline void plan_tasks(StageArgs &A, int64_t units, int64_t wave, double start, double idle, int free = 12)
 {
     A.R = 1;
     A.ntasks = A.ngroups;
@@ -130,12 +142,16 @@ inline void plan_tasks(StageArgs &A, int64_t units, int64_t wave, double start, 
     // autotuner's candidates, 7.48 with its own pick). So are the groups of several chunks in one launch.
     if (A.nseg > 1 || A.fixed)
         return;
-    auto last = [&](double x) { return x > 0.0 ? idle + (1.0 - idle) * x : 0.0; };
     double best = 0.0;
     for (int r = 1; r <= A.ngroups; r++) {
         const int tasks = (A.ngroups + r - 1) / r;
         const double len = (double)(r * A.G < A.nvt ? r * A.G : A.nvt) + start;
         const double rounds = (double)(units * tasks) / (double)wave, part = rounds - (double)(int64_t)rounds;
+        const double q = rounds < kRounds ? kIdleFew : idle;
+        auto last = [q](double x) { return x > 0.0 ? q + (1.0 - q) * x : 0.0; };
+        const bool one = A.G <= 2 && rounds > 0.9 && rounds <= 1.0;
+        if (r > 1 && r * A.G > free && rounds < kRounds && !one)
+            continue;
         const double cost = rounds <= 1.0 ? 1.1 * last(rounds) * len  // (nothing left to balance the SMs with)
                                           : units * (A.nvt + start * tasks) / (double)wave + (last(part) - part) * len;
         if (r == 1 || cost < best) {

@@ -1335,7 +1335,7 @@ cudaError_t launch3c(const StageArgs &A0, cudaStream_t s)
                           offsetof(Sm, fnm) % 16 == 0 && offsetof(Sm, fpar) % 16 == 0 && offsetof(Sm, lim) % 16 == 0 &&
                           offsetof(Sm, bar) % 8 == 0,
                       "8- and 16-byte shared accesses");
-        plan_tasks(A, A.mesh.nelem, 152 * 16, 0.8, 0.5);
+        plan_tasks(A, A.mesh.nelem, 152 * 16, 0.8, 0.5, 8);  // (12 free tiles: up to 1.24 of single groups' time)
         k_stage3cp<N1, GEN><<<A.mesh.nelem * A.ntasks, kWarp * N1 / 2, sizeof(Sm), s>>>(A);
     } else {
         plan_tasks(A, A.mesh.nelem, 152 * (N1 >= 4 ? BGK_STAGE3C_MINCTAS_P3 : 6), 0.8, 0.6);
