@@ -12,6 +12,10 @@
 #ifndef BGK_STAGE3W_MINCTAS_P2
 #define BGK_STAGE3W_MINCTAS_P2 13  // resident CTAs per SM the register allocation is sized for (p = 2)
 #endif
+// At p = 1 the periodic and the Dirichlet-and-limiter form fit 96 registers and so 20 one-warp CTAs; left to itself the
+// compiler took 104 for the latter, which leaves 16 (every quarter of an SM loses one): 17 x 22 x 15 elements of 24^3
+// velocities 261 -> 246 us per launch, 18 x 19 x 14 without limiter 212 -> 202 with the group index kept (both with the
+// task rule's change).
 
 namespace bgk {
 
@@ -48,7 +52,7 @@ struct __align__(16) Stage3wWarp {  // a multiple of 16 bytes, so every warp's c
 };
 
 template <int N1, int OCT, int GEN>
-__global__ void __launch_bounds__(kWarp *BGK_STAGE3W_WARPS, (N1 == 3 ? BGK_STAGE3W_MINCTAS_P2 : 16))
+__global__ void __launch_bounds__(kWarp *BGK_STAGE3W_WARPS, (N1 == 3 ? BGK_STAGE3W_MINCTAS_P2 : (GEN == 1 ? 16 : 20)))
     k_stage3w(const StageArgs A)
 {
     constexpr int NQ = N1 * N1;
@@ -69,6 +73,8 @@ __global__ void __launch_bounds__(kWarp *BGK_STAGE3W_WARPS, (N1 == 3 ? BGK_STAGE
     int vl0, vl1;
     task_tiles(A, gl, vl0, vl1);
     int ge = min(vl0 + A.G, vl1);  // end of the moment group
+    // its index: kept at p = 1, whose groups are short beside the divisions that form it again (p = 2 has no register left)
+    int grp = N1 == 2 ? A.group0 + (A.nseg == 1 ? gl * A.R : gl) : 0;
     int ec[3];
     ec[0] = e % A.mesh.ne[0];
     ec[1] = (e / A.mesh.ne[0]) % A.mesh.ne[1];
@@ -475,7 +481,8 @@ __global__ void __launch_bounds__(kWarp *BGK_STAGE3W_WARPS, (N1 == 3 ? BGK_STAGE
             ka = ka == 2 ? 0 : ka + 1;
         }
         // the end of a moment group: combine the 4 velocity eighths of every row
-        const int grp = moment_group(A, blockIdx.x / nblk, vl - 1);
+        if (N1 != 2)
+            grp = moment_group(A, blockIdx.x / nblk, vl - 1);
 #pragma unroll
         for (int h = 0; h < NHR; h++) {
             const int q = np + 8 * h;
@@ -490,6 +497,8 @@ __global__ void __launch_bounds__(kWarp *BGK_STAGE3W_WARPS, (N1 == 3 ? BGK_STAGE
             }
         }
         ge = min(ge + A.G, vl1);
+        if (N1 == 2)
+            grp++;
     }
 }
 
