@@ -11,6 +11,7 @@
 // A stage reads neighbours only inside its own chunk, and chunks run in order on one stream, so a
 // slot is rewritten only after the launch that read it has finished. Memory = A + (C+1)/C arrays.
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -74,11 +75,8 @@ bool reserve_merge_extra(int64_t bytes)
     } while (!g_merge_extra.compare_exchange_weak(held, held + bytes));
     return true;
 }
-// Tiles per task of the batched line launches (whole moment groups of at least this, see batch_upload)
-#ifndef BGK_BATCH_TILES
-#define BGK_BATCH_TILES 16
-#endif
-const int kBatchTiles = BGK_BATCH_TILES;
+// Longest task, in tiles, of the batched line launches where the library chooses (see batch_tiles)
+const int kBatchTiles = 16;
 const int kMinTuneG = 2;  // shortest task (tiles per warp task) the autotuner tries
 
 struct Chunk {
@@ -1972,13 +1970,32 @@ int bfail(bgk_batch *b, int code, const std::string &msg)
             return bfail(b, BGK_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
+// Tiles per task of a batch's members by degree (one launch each): one for every seven rounds that single-tile tasks
+// would make on the resident warps, up to kBatchTiles. Longer tasks spare set-up, and in a small batch leave the
+// chip idle. Members of the Sod ensemble's ranges, degrees 1 to 3, us per step with at least 1 / 4 / 8 / 16 tiles per
+// task: 2 members 147 / 215 / 287 / 397, 4 members 188 / 289 / 382 / 589, 16 members 613 / 654 / 739 / 929, 64 members
+// 1544 / 1487 / 1464 / 1578, 256 members 4907 / 4730 / 4698 / 4651.
+std::array<int, kMaxN1 + 1> batch_tiles(const bgk_batch *b)
+{
+    std::array<int64_t, kMaxN1 + 1> work{};
+    std::array<int, kMaxN1 + 1> tiles{};
+    for (bgk_ctx *c : b->probs) {
+        StageArgs A = stage_args(c, c->chunks[0]);
+        A.ntasks = 1;
+        work[c->N1] += (int64_t)stage1d_batch_tasks(A) * A.nvt;
+    }
+    for (int n1 = 0; n1 <= kMaxN1; n1++)
+        tiles[n1] = (int)std::max<int64_t>(1, std::min<int64_t>(kBatchTiles, work[n1] / (7 * 152 * 12)));
+    return tiles;
+}
+
 // Member c's stage arguments in a batch (the caller sets the buffers and the step): its one chunk, in tasks of
-// at least kBatchTiles tiles unless its length was given or measured. The task table and bgk_batch_info both count
-// these tasks.
-StageArgs batch_member_args(bgk_ctx *c)
+// whole moment groups of about `tiles` tiles unless its length was given or measured. The task table and
+// bgk_batch_info both count these tasks.
+StageArgs batch_member_args(bgk_ctx *c, int tiles)
 {
     StageArgs A = stage_args(c, c->chunks[0]);
-    A.R = A.fixed ? 1 : std::max(1, kBatchTiles / A.G);
+    A.R = A.fixed ? 1 : std::max(1, tiles / A.G);
     A.ntasks = (A.ngroups + A.R - 1) / A.R;
     return A;
 }
@@ -1991,6 +2008,7 @@ int batch_upload(bgk_batch *b, const double *dt)
     std::vector<StageArgs> sa(3 * (size_t)n);
     std::vector<NewtonArgs> na(n);
     std::vector<int> ts(n + 1, 0), ps(n + 1, 0);
+    const auto tiles = batch_tiles(b);
     for (int s = 0; s < 3; s++)
         b->alg_bytes[s] = 0.0;
     for (int q = 0; q < n; q++) {
@@ -2000,7 +2018,7 @@ int batch_upload(bgk_batch *b, const double *dt)
         for (int v = 0; v < c->nslots; v++)
             real += c->slotk[v] >= 0;
         for (int st = 0; st < 3; st++) {
-            StageArgs A = batch_member_args(c);
+            StageArgs A = batch_member_args(c, tiles[c->N1]);
             A.src = st == 0 ? Aq : (st == 1 ? s1 : s2);
             A.fn = st == 0 ? nullptr : Aq;
             A.dst = st == 0 ? s1 : (st == 1 ? s2 : Aq);
@@ -2373,10 +2391,11 @@ int bgk_batch_info(const bgk_batch *b, int64_t *npoints, int64_t *ndof, int64_t 
     if (!b)
         return BGK_EINVAL;
     int64_t np = 0, nd = 0, nt = 0;
+    const auto tiles = batch_tiles(b);
     for (const bgk_ctx *c : b->probs) {
         np += c->npts;
         nd += c->npts * c->nvel;
-        nt += stage1d_batch_tasks(batch_member_args(const_cast<bgk_ctx *>(c)));
+        nt += stage1d_batch_tasks(batch_member_args(const_cast<bgk_ctx *>(c), tiles[c->N1]));
     }
     if (npoints)
         *npoints = np;
