@@ -2,10 +2,10 @@
 // form, FP32-split, its batched persistent variant, and the dispatch of all stage kernels.
 //
 // One task = a run of consecutive elements x a run of velocity tiles (32 velocities of one sign octant each),
-// on one warp: for p <= 3 half-warps of 16 nodes and packed pairs of velocities (line_task_pair), else and in
-// the moments-only pass 16 nodes and a lane per velocity (line_task). The warp streams its tiles through two
-// shared buffers with bulk asynchronous copies on its own mbarriers, one tile ahead, and shares no barrier
-// with any other warp.
+// on one warp: for p <= 3 half-warps of 16 nodes and packed pairs of velocities (line_task_pair), else, in launches
+// of few tasks and in the moments-only pass 16 nodes and a lane per velocity (line_task). The warp streams its
+// tiles through two shared buffers with bulk asynchronous copies on its own mbarriers, one tile ahead, and shares
+// no barrier with any other warp.
 //
 // The stage never reads what another task of the same launch writes: it reads f_s (source), f^n,
 // the BGK exponent table and the ghost table, and writes only its own part of the destination and
@@ -825,10 +825,16 @@ template <int N1>
 static cudaError_t launch_1d(const StageArgs &A0, int mode, cudaStream_t s)
 {
     StageArgs A = A0;
-    if constexpr (N1 <= 4) {  // p <= 3: packed pairs of velocities (the moments-only pass keeps the lane per velocity)
-        if (mode == 0) {
-            constexpr int K2 = 2 * LinePair<N1>::KH;
-            plan_tasks(A, (A.mesh.nelem + K2 - 1) / K2, 152 * kLinePairCtas * kLinePairWarps, 0.8, 0.75);
+    if constexpr (N1 <= 4) {
+        // p <= 3: packed pairs of velocities, where their tasks, twice as long, fill half of a round or more (counted in
+        // tiles: a short last group fills little). Below, the lane per velocity (and in the moments-only pass). us per
+        // launch, pairs against it: 629 elements, p = 1, 28^3 velocities (0.24 of a round) 21.2 and 20.6; 948, p = 2, 24^3
+        // (0.36) 24.8 and 22.9; 1902, p = 3, 18^3 (0.39) 24.9 and 23.0; 1018, p = 3, 24^3 (0.47) 26.5 and 24.4; 3353, p = 2,
+        // 18^3 (0.53) 25.3 and 26.2; 4300 (0.68) 30.6 and 34.4.
+        constexpr int K2 = 2 * LinePair<N1>::KH;
+        const int64_t runs = (A.mesh.nelem + K2 - 1) / K2, wave = 152 * kLinePairCtas * kLinePairWarps;
+        if (mode == 0 && 2 * runs * A.nvt >= wave * A.G) {
+            plan_tasks(A, runs, wave, 0.8, 0.75);
             k_stage1d_pair<N1><<<(pair_tasks<N1>(A) + kLinePairWarps - 1) / kLinePairWarps, kWarp * kLinePairWarps,
                                  kLinePairWarps * sizeof(LinePair<N1>), s>>>(A);
             return cudaGetLastError();
@@ -837,11 +843,9 @@ static cudaError_t launch_1d(const StageArgs &A0, int mode, cudaStream_t s)
     plan_line<N1>(A);
     const int ctas = (line_tasks<N1>(A) + BGK_LINE_WARPS - 1) / BGK_LINE_WARPS;
     const size_t smem = BGK_LINE_WARPS * sizeof(LineWarp<N1>);
-    if constexpr (N1 > 4) {
-        if (mode == 0) {
-            k_stage1d<N1, 0><<<ctas, kWarp * BGK_LINE_WARPS, smem, s>>>(A);
-            return cudaGetLastError();
-        }
+    if (mode == 0) {
+        k_stage1d<N1, 0><<<ctas, kWarp * BGK_LINE_WARPS, smem, s>>>(A);
+        return cudaGetLastError();
     }
     k_stage1d<N1, 1><<<ctas, kWarp * BGK_LINE_WARPS, smem, s>>>(A);
     return cudaGetLastError();
