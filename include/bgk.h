@@ -99,7 +99,9 @@ typedef struct {
                                 contexts together hold at most 1 GiB beyond the rotating ones) and one after
                                 the other on rotating buffers elsewhere; any other value always one after the
                                 other. The results do not depend on how the octants are launched. */
-    int vtiles_per_task;     /* 32-velocity tiles per warp task, 0 = automatic */
+    int vtiles_per_task;     /* 32-velocity tiles per warp task and moment group, 0 = automatic (groups of at most 8
+                                tiles, tasks of one or more groups). A given length is kept; long ones leave the chip
+                                idle on a mesh of few elements. */
     int maxwellian;          /* BGK_MAXWELLIAN_CONSERVATIVE (0, the method) or BGK_MAXWELLIAN_CONTINUOUS
                                 (the ablation: g = the sampled continuous Maxwellian of the moments, whose
                                 discrete moments differ from them, Sec. 2.1, Eq. 13) */

@@ -7,7 +7,7 @@
 //   stage 1: chunk c reads A[c]                      -> writes slot c
 //   stage 2: chunk c reads slot c (+ A[c])           -> writes slot c-1 (slot C for c = 0)
 //   stage 3: chunk c reads its stage-2 slot (+ A[c]) -> writes A[c] in place
-// (a small problem instead keeps two full stage buffers and launches all chunks of a stage together)
+// (a small problem instead keeps two full stage buffers and launches all chunks of a stage together: 3 arrays)
 // A stage reads neighbours only inside its own chunk, and chunks run in order on one stream, so a
 // slot is rewritten only after the launch that read it has finished. Memory = A + (C+1)/C arrays.
 #include <algorithm>

@@ -330,7 +330,8 @@ __device__ __forceinline__ void line_task(const StageArgs &A, const int task, co
 // their order are those of line_task. A warp then runs twice the elements per instruction and reads the
 // exponents (a shared load returns 128 bytes per cycle, broadcast or not) once per 64 velocities. f_s is
 // double-buffered between the rows of the run's two outside neighbours (only the upwind one is copied), f^n
-// single (the next tile's lands once this tile's is in registers). Bound: latency and issue at 12 warps per SM.
+// single (the next tile's lands once this tile's is in registers). Bound: latency and issue at 12 warps per SM
+// (launches of fewer tasks: launch_1d).
 // 65,536 elements at p = 3, 32^2 velocities: 0.148 -> 0.127 ms per octant launch (5.7 TB/s); 60,001 at p = 1,
 // 40^2 velocities, three steps 7.78 -> 4.02 ms; four steps of the Sod ensemble with their sampling 26.7 -> 24.8.
 // ------------------------------------------------------------------------------------------------
@@ -863,7 +864,7 @@ cudaError_t prepare_stage(int dim, int p)
     } else if (dim == 1 && p >= 1 && p <= 5) {
         return cudaSuccess;  // the line kernels stay within the default dynamic shared memory
     } else if (dim == 2 && p >= 1 && p <= 3) {
-        return cudaSuccess;  // the quadrilateral kernels use static shared memory only
+        return cudaSuccess;  // as do the quadrilateral ones (k_stage2 static, k_stage2p dynamic)
     }
     return cudaErrorInvalidValue;
 }

@@ -708,9 +708,9 @@ __global__ void __launch_bounds__(kWarp *N1, (N1 >= 4 ? BGK_STAGE3C_MINCTAS_P3 :
 // face normal or an exponent that a lane reads for one velocity costs as much as its share of f; a lane with
 // two velocities halves that, and one warp holds the element. 16 x 12 x 14 elements, p = 1, 24^3 velocities,
 // two steps: 15.8 -> 10.8 ms. At p = 3 it runs too, but slower (2.08 -> 2.35 ms per octant launch of
-// 16^3 elements, 24^3 velocities: 92 instructions per 32 degrees of freedom at 0.4 per cycle; its 168
-// registers leave 10 warps per SM, and its code overflows the instruction cache), so p = 3 stays with the
-// lane per velocity.
+// 16^3 elements, 24^3 velocities: 92 instructions per 32 degrees of freedom at 0.4 per cycle; its 41 KB of
+// shared memory leave 5 CTAs, 10 warps per SM, where its 168 registers would allow 6, and its code overflows the
+// instruction cache), so p = 3 stays with the lane per velocity. A form in less shared memory was not tried.
 // ------------------------------------------------------------------------------------------------
 constexpr bool stage3c_pairs(int N1) { return N1 == 2; }
 
@@ -1278,7 +1278,9 @@ __global__ void __launch_bounds__(kWarp *N1 / 2, 16) k_stage3cp(const StageArgs 
             fence_proxy_async();
             issue(ys, vl + 1, bF);
         }
-        if (vl + 1 == ge) {  // the end of a moment group: combine the 4 velocity eighths of a row
+        // the end of a moment group: combine the 4 velocity eighths of a row (in the tile loop, as it was first written;
+        // outside it, as in k_stage3s, it was not measured here)
+        if (vl + 1 == ge) {
             const int grp = moment_group(A, blockIdx.x / E, vl);
             ge = min(ge + A.G, vl1);
 #pragma unroll

@@ -18,7 +18,7 @@ namespace bgk {
 // moved to form a pair, and an instruction covers 64 degrees of freedom. Each half performs the scalar
 // form's operations in its order.
 // Bound: the latency of the dependent FP32 pairs and shared loads at 12 warps per SM (issue slots half used),
-// with shared memory's data path close behind: per 32 degrees of freedom it takes 18 cycles for the copies
+// with shared memory's data path close behind: per 32 degrees of freedom it takes 19.5 cycles for the copies
 // in (5), the lines (8), the exponents (4: a load returns 128 bytes per cycle, broadcast or not) and the
 // moments (2.5) of the 27 that a launch takes. A lane per velocity with packed pairs of lines (four warps
 // per element) read the exponents once per 32 velocities (8 cycles) and took 70 instructions per 32 degrees
