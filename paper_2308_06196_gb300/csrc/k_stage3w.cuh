@@ -74,7 +74,9 @@ __global__ void __launch_bounds__(kWarp *BGK_STAGE3W_WARPS, (N1 == 3 ? BGK_STAGE
     task_tiles(A, gl, vl0, vl1);
     int ge = min(vl0 + A.G, vl1);  // end of the moment group
     // its index: kept at p = 1, whose groups are short beside the divisions that form it again (p = 2 has no register left)
-    int grp = N1 == 2 ? A.group0 + (A.nseg == 1 ? gl * A.R : gl) : 0;
+    [[maybe_unused]] int grp2 = 0;
+    if constexpr (N1 == 2)
+        grp2 = A.group0 + (A.nseg == 1 ? gl * A.R : gl);
     int ec[3];
     ec[0] = e % A.mesh.ne[0];
     ec[1] = (e / A.mesh.ne[0]) % A.mesh.ne[1];
@@ -481,8 +483,7 @@ __global__ void __launch_bounds__(kWarp *BGK_STAGE3W_WARPS, (N1 == 3 ? BGK_STAGE
             ka = ka == 2 ? 0 : ka + 1;
         }
         // the end of a moment group: combine the 4 velocity eighths of every row
-        if (N1 != 2)
-            grp = moment_group(A, blockIdx.x / nblk, vl - 1);
+        const int grp = N1 == 2 ? grp2 : moment_group(A, blockIdx.x / nblk, vl - 1);
 #pragma unroll
         for (int h = 0; h < NHR; h++) {
             const int q = np + 8 * h;
@@ -497,8 +498,8 @@ __global__ void __launch_bounds__(kWarp *BGK_STAGE3W_WARPS, (N1 == 3 ? BGK_STAGE
             }
         }
         ge = min(ge + A.G, vl1);
-        if (N1 == 2)
-            grp++;
+        if constexpr (N1 == 2)
+            grp2++;
     }
 }
 
