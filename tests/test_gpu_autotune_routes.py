@@ -24,6 +24,6 @@ def test_each_launch_form_is_tuned(first):
         return time.perf_counter() - t
 
     tuned(first)
-    other, repeat = tuned(8 - first), tuned(first)
+    other, repeat = tuned(8 - first), min(tuned(first) for _ in range(4))
     # some ten lengths, three stage passes of 20 us or more each, against a look into the cache
     assert other > 3e-4 and other > 5 * repeat, (other, repeat)
